@@ -236,7 +236,8 @@ rcm_status rcm_order_batch(int32_t G, int64_t n_total, const int64_t *goff, cons
 /* Tuning of the batched path (apart from row_order, every value gives the same permutations;
    only speed differs). */
 typedef struct {
-    int32_t block_threads;   /* threads per CTA of the batched executor: 128, 256 or 512; 0 = 256   */
+    int32_t block_threads;   /* threads per CTA of the batched executor: 128, 256 or 512; 0 = from
+                                the graphs' sizes (wide CTAs for few graphs, narrow for many)      */
     int32_t row_sort_split;  /* rows with at most this many stored entries are sorted by one thread,
                                 longer rows by a whole CTA: 4..32; 0 = 32                          */
     int32_t row_order;       /* as rcm_options.row_order: 1 = sort-free variant (changes the result) */

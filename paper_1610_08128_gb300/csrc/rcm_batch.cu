@@ -15,20 +15,56 @@
 
 namespace rcm {
 
-constexpr int kBatchSortCap = 2048;  // component tables sorted in shared memory up to this size
+// Hash slots of the local sweeps: levels of up to about 1,500 new vertices.
+constexpr int kBatchSlots = 2048;
+constexpr int kBatchEntries = 3072;          // list entries of all warps
+constexpr int kBatchStaticSmem = 20 * 1024;  // EngineSmem and the rest, rounded up
+constexpr int kSmemPerSm = 227 * 1024;
 
-// CTAs per SM the batched executor is compiled for: many graphs are small, so occupancy matters
-// more than registers (256 threads: 3 per SM at 80 registers measured faster than 4 at 64).
+// Largest graph whose bitmap fits when the launch's G graphs want up to batch_min_blocks CTAs on an SM.
+static int local_cap_for(int max_n, int G, int per_sm, int sms) {
+    const int want = std::max(1, std::min(per_sm, (G + sms - 1) / sms));
+    const long long bytes = kSmemPerSm / want - 1024 - kBatchStaticSmem - (long long)local_bytes(0, kBatchSlots, kBatchEntries);
+    return (int)std::min<long long>(max_n, std::max<long long>(0, bytes / 16 * 128));
+}
+
+// CTAs per SM the batched executor is compiled for: 128 registers at every width. A level's time is
+// the latency of one warp's instructions; with 64 or 80 registers the local sweeps lose the overlap of
+// their loads (500 graphs of up to 50,000 vertices on 256-thread CTAs: 3.2 ms with 128 registers, 4.2
+// with 80; 10,000 of them on 128-thread CTAs: 13.7 ms with 4 CTAs on an SM, 15.0 with 5, 17.8 with 8).
 template <int kThreads>
-constexpr int batch_min_blocks() { return kThreads >= 512 ? 2 : kThreads >= 256 ? 3 : 5; }
+constexpr int batch_min_blocks() { return kThreads < 512 ? 512 / kThreads : 1; }
+
+// CTA width when the caller names none. Wide CTAs finish a graph sooner, narrow ones order more
+// vertices per SM: a batch takes about the larger of tail x (vertices of its largest graph) and
+// rate x (all its vertices). Nanoseconds per vertex on GB300 (mixes of grids and meshes, log-uniform
+// sizes); 10,000 graphs up to 50,000 vertices: 13.7 / 17.7 / 26.0 ms on 128 / 256 / 512 threads; 4,000:
+// 10.0 / 7.1 / 10.4; 1,000: 7.9 / 4.8 / 3.4; 400 up to 200,000: 20.1 / 11.0 / 7.3.
+static int batch_threads(long long n_total, int max_n) {
+    static const struct { int threads; double tail, rate; } kWidths[] = {
+        {128, 160.0, 0.17}, {256, 95.0, 0.22}, {512, 57.0, 0.32}};
+    int best = 256;
+    double least = 1e300;
+    for (const auto& w : kWidths) {
+        const double t = std::max(w.tail * max_n, w.rate * (double)n_total);
+        if (t < least) {
+            least = t;
+            best = w.threads;
+        }
+    }
+    return best;
+}
 
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads, batch_min_blocks<kThreads>()) k_rcm_batch(BatchArgs b) {
+    // the local sweeps' state (rcm_local.cuh); component tables sort in the same bytes
+    extern __shared__ __align__(16) unsigned s_local[];
     __shared__ EngineSmem smem;
     __shared__ int s_item;
-    __shared__ unsigned long long s_sort[kBatchSortCap + kBatchSortCap / 2];
     if (ld_volatile(&b.ctl->status) & kErrBadCsr) return;
     Engine<true> e;
+    const int sort_cap = (int)(local_bytes(b.local_cap, b.local_slots, b.local_entries) / 12);
+    if (threadIdx.x == 0) local_init(&smem.loc, b.local_cap, b.local_slots, b.local_entries, s_local);
     while (true) {
         if (threadIdx.x == 0) s_item = atomicAdd(&b.ctl->work_next, 1);
         __syncthreads();
@@ -82,8 +118,8 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks<kThreads>()) k_rcm_
         a.mid_thr = 0;
         __syncthreads();
         e.init(a, &smem);
-        e.sm_sort = s_sort;
-        e.sm_sort_cap = kBatchSortCap;
+        e.sm_sort = (unsigned long long*)s_local;
+        e.sm_sort_cap = sort_cap;
         if (!e.run()) return;
         __syncthreads();
         // the segment holds global ids while running; the result is in local ids
@@ -129,6 +165,13 @@ std::vector<int> batch_order(const std::vector<long long>& goff) {
     return order;
 }
 
+// Vertices of the largest graph.
+static int batch_max(const std::vector<long long>& goff) {
+    long long m = 0;
+    for (size_t i = 0; i + 1 < goff.size(); ++i) m = std::max(m, goff[i + 1] - goff[i]);
+    return (int)std::min<long long>(std::max<long long>(m, 0), kIntMax);
+}
+
 static std::mutex g_batch_mu;
 static int g_batch_per_sm[3] = {-1, -1, -1};  // CTAs per SM of the 128-, 256- and 512-thread executor
 
@@ -148,7 +191,9 @@ static int batch_blocks_per_sm(int threads) {
     std::lock_guard<std::mutex> g(g_batch_mu);
     if (g_batch_per_sm[idx] < 0) {
         int bps = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, batch_kernel(threads), threads, 0);
+        const void* k = batch_kernel(threads);
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm - kBatchStaticSmem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, threads, local_bytes(0, kBatchSlots, kBatchEntries));
         g_batch_per_sm[idx] = bps;
         cudaFuncSetAttribute(k_sort_rows_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(sizeof(unsigned long long) * kBigRowSmem));
@@ -158,13 +203,14 @@ static int batch_blocks_per_sm(int threads) {
 
 rcm_status batch_tuning(const rcm_batch_options* o, BatchTuning* out) {
     BatchTuning t;
+    t.threads = 0;
     if (o) {
         if (o->block_threads) t.threads = o->block_threads;
         if (o->row_sort_split) t.small_max = o->row_sort_split;
         if (o->row_order != 0 && o->row_order != 1) return RCM_ERR_INVALID_ARG;
         t.by_degree = o->row_order ? 0 : 1;
     }
-    if (batch_index(t.threads) < 0 || t.small_max < 4 || t.small_max > kSmallRowMax) return RCM_ERR_INVALID_ARG;
+    if ((t.threads && batch_index(t.threads) < 0) || t.small_max < 4 || t.small_max > kSmallRowMax) return RCM_ERR_INVALID_ARG;
     *out = t;
     return RCM_OK;
 }
@@ -176,7 +222,7 @@ bool batch_prepare(const BatchTuning& t) {
 
 cudaError_t enqueue_batch(int G, long long n_total, int nnz, const long long* goff, const int* order,
                           const int* rowptr, const int* colidx, int* perm, char* base, const BatchLayout& L,
-                          const BatchTuning& t, cudaStream_t s) {
+                          const BatchTuning& t, cudaStream_t s, int max_n) {
     const DeviceInfo& di = device_info();
     const int per_sm = batch_blocks_per_sm(t.threads);
     if (per_sm <= 0) return cudaErrorInvalidConfiguration;
@@ -224,9 +270,15 @@ cudaError_t enqueue_batch(int G, long long n_total, int nnz, const long long* go
     b.cc_gkey = (unsigned long long*)(base + L.ccgk);
     b.cc_gidx = (int*)(base + L.ccgi);
     b.cc_tab = (int4*)(base + L.cct);
-    const int blocks = (int)std::min<long long>((long long)per_sm * di.sms, std::max(G, 1));
+    b.local_cap = local_cap_for(max_n, G, per_sm, di.sms);
+    b.local_slots = kBatchSlots;
+    b.local_entries = kBatchEntries;
+    const size_t smem = local_bytes(b.local_cap, b.local_slots, b.local_entries);
+    // at most as many CTAs as the local state leaves room for (more would only wait)
+    const long long fit = std::max<long long>(1, std::min<long long>(per_sm, kSmemPerSm / (long long)(smem + kBatchStaticSmem + 1024)));
+    const int blocks = (int)std::min<long long>(fit * di.sms, std::max(G, 1));
     void* kargs[] = {&b};
-    return cudaLaunchKernel(batch_kernel(t.threads), dim3(blocks), dim3(t.threads), kargs, 0, s);
+    return cudaLaunchKernel(batch_kernel(t.threads), dim3(blocks), dim3(t.threads), kargs, smem, s);
 }
 
 rcm_status order_batch(int32_t G, int64_t n_total, const int64_t* goff, const int32_t* rowptr,
@@ -234,7 +286,6 @@ rcm_status order_batch(int32_t G, int64_t n_total, const int64_t* goff, const in
     BatchTuning t;
     rcm_status st = batch_tuning(opts, &t);
     if (st != RCM_OK) return st;
-    if (!batch_prepare(t)) return RCM_ERR_CUDA;
     // nnz sizes the sorted-adjacency copy and the graph sizes set the work-queue order: one
     // synchronised read of rowptr[n_total] and goff
     int nnz = 0;
@@ -245,6 +296,9 @@ rcm_status order_batch(int32_t G, int64_t n_total, const int64_t* goff, const in
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_status(e);
     if (nnz < 0) return RCM_ERR_BAD_CSR;
+    const int max_n = batch_max(goff_h);
+    if (t.threads == 0) t.threads = batch_threads(n_total, max_n);
+    if (!batch_prepare(t)) return RCM_ERR_CUDA;
     const BatchLayout L = batch_layout(n_total, nnz, G);
     int* latch = stream_latch(s);
     if (!latch) return RCM_ERR_TOO_LARGE;  // every latch slot held by streams whose status is unread
@@ -257,7 +311,7 @@ rcm_status order_batch(int32_t G, int64_t n_total, const int64_t* goff, const in
     e = cudaMemcpyAsync(base + L.order, order.data(), sizeof(int) * (size_t)G, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = enqueue_batch(G, n_total, nnz, (const long long*)goff, (const int*)(base + L.order), rowptr, colidx,
-                          perm, base, L, t, s);
+                          perm, base, L, t, s, max_n);
     if (e == cudaSuccess) e = enqueue_latch((Ctl*)(base + L.ctl), latch, nullptr, s);
     ws_free(ws, s);
     return e == cudaSuccess ? RCM_OK : cuda_status(e);
@@ -276,7 +330,6 @@ rcm_status batch_plan_create(int32_t G, int64_t n_total, int64_t nnz, const int6
     BatchTuning t;
     rcm_status st = batch_tuning(opts, &t);
     if (st != RCM_OK) return st;
-    if (!batch_prepare(t)) return RCM_ERR_CUDA;
     BatchPlan* p = new (std::nothrow) BatchPlan();
     if (!p) return RCM_ERR_OOM;
     const BatchLayout L = batch_layout(n_total, nnz, G);
@@ -284,6 +337,9 @@ rcm_status batch_plan_create(int32_t G, int64_t n_total, int64_t nnz, const int6
     // work-queue order (largest graph first) from the graph offsets at creation
     std::vector<long long> goff_h((size_t)G + 1);
     if (e == cudaSuccess) e = cudaMemcpy(goff_h.data(), goff, sizeof(long long) * goff_h.size(), cudaMemcpyDeviceToHost);
+    const int max_n = batch_max(goff_h);
+    if (t.threads == 0) t.threads = batch_threads(n_total, max_n);
+    if (e == cudaSuccess && !batch_prepare(t)) e = cudaErrorInvalidConfiguration;
     if (e == cudaSuccess) {
         const std::vector<int> order = batch_order(goff_h);
         e = cudaMemcpy((char*)p->ws + L.order, order.data(), sizeof(int) * (size_t)G, cudaMemcpyHostToDevice);
@@ -294,7 +350,7 @@ rcm_status batch_plan_create(int32_t G, int64_t n_total, int64_t nnz, const int6
     if (e == cudaSuccess) {
         const cudaError_t ee = enqueue_batch(G, n_total, (int)nnz, (const long long*)goff,
                                              (const int*)((char*)p->ws + L.order), rowptr, colidx, perm,
-                                             (char*)p->ws, L, t, cs);
+                                             (char*)p->ws, L, t, cs, max_n);
         e = cudaStreamEndCapture(cs, &p->graph);
         if (e == cudaSuccess) e = ee;
     }

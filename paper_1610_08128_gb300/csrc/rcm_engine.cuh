@@ -44,105 +44,11 @@
 #pragma once
 
 #include "rcm_cc.cuh"
+#include "rcm_engine_state.cuh"
 #include "rcm_internal.cuh"
+#include "rcm_local.cuh"
 
 namespace rcm {
-
-constexpr int kEllNb = 7;       // neighbours stored in a vertex's 32-byte row; slot 7 = degree
-constexpr int kCache = 2048;    // frontier ids cached in shared memory per buffer
-constexpr int kTinyMax = 32;    // components of at most this many vertices are ordered by one thread
-constexpr int kWarpLevel = 32;  // narrow levels of at most this many vertices run on warp 0 alone
-// A level of a few hundred vertices that holds a hub is far more work than one CTA does quickly,
-// and a labelled first sweep over hubs costs more than a levels-only one: graphs with a vertex of
-// more than kHubDegree neighbours take a lower frontier switch and levels-only first sweeps by
-// default (the 1M-vertex power-law graph with hubs of 7,000: 24.3 ms with the grid defaults,
-// 8.8 ms with these).
-constexpr int kHubDegree = 512;
-constexpr int kHubNarrow = 128;
-constexpr unsigned long long kClaimNone = ~0ull;
-
-struct EngineArgs {
-    int n;                       // vertices of this graph
-    int v0;                      // global id of its first vertex (rows hold global ids)
-    const int* rowptr;           // global rows (overflow neighbours of rows with degree > 7)
-    const int4* ell;             // 2 x int4 per vertex: 7 sorted neighbours (-1 padded) + degree
-    const int* adj;              // full sorted rows, valid for rows with degree > 7
-    const int* deg;              // global
-    unsigned long long* claim;   // global, 64-bit keys (kClaimNone = not reached)
-    int* vis;                    // global sweep stamps
-    int* qa;                     // this graph's queue / staging buffer (n ints)
-    int* qb;                     // this graph's queue / staging buffer (n ints)
-    int* boff;                   // this graph's per-frontier offsets (n ints)
-    int* perm;                   // this graph's output segment (n ints); global ids while running
-    Ctl* ctl;                    // grid control block (whole-grid executor only)
-    int* status;                 // where device-detected error bits are ORed
-    int* diag;                   // optional (may be null): first failed guard's site and value
-    int narrow_thr;
-    int fused;
-    int cc_first;                // persistent grid: build the component table before the first sweep
-    int hub_auto;                // default launch of the persistent grid: a graph with a vertex of more
-                                 // than kHubDegree neighbours takes the frontier switch kHubNarrow and
-                                 // levels-only first sweeps (decided on the device from ctl->maxdeg)
-    int obits;                   // low bits of a key holding the in-level order
-    int profile;                 // accumulate per-phase time (CTA 0, thread 0)
-    long long limit_ns;
-    // concurrent components (whole-grid executor only)
-    int* cc_parent;              // n ints
-    int* cc_size;                // n ints (indexed by root)
-    unsigned long long* cc_key;  // n keys (indexed by root)
-    int* cc_roots;               // cc_cap ints
-    unsigned long long* cc_gkey; // next_pow2(cc_cap) keys (sort scratch beyond shared memory)
-    int* cc_gidx;                // next_pow2(cc_cap) ints
-    int4* cc_tab;                // cc_cap entries: (start vertex, first label, size, root)
-    int cc_cap;                  // most components ordered concurrently (else one by one)
-    int cc_big;                  // components at least this large run on the whole grid
-    // bottom-up expansion (whole-grid executor only; fkey == null: top-down only)
-    unsigned long long* fkey;    // n words: a labelled frontier vertex's key, published for bottom-up claims
-    int expand_mode;             // 2 = bottom-up on every grid level, 1 = top-down, else per level by frontier size
-    int bu_divisor;              // per level: bottom-up once the frontier holds n / bu_divisor vertices
-    // asynchronous levels-only sweeps (whole-grid executor only; adist == null: level by level)
-    unsigned long long* adist;   // n words: (~sweep stamp) << 32 | breadth-first distance
-    unsigned long long* aq;      // work queue of aq_cap (distance << 32 | vertex) items
-    AsyncCtl* actl;
-    unsigned aq_cap;
-    // middle tier (whole-grid executor launched in clusters of mid_k CTAs; 0 = off): labelled
-    // levels of narrow_thr <= size < mid_thr run on cluster 0 alone, exchanging through
-    // distributed shared memory, while the other CTAs wait at the next grid barrier
-    int mid_k;
-    int mid_thr;
-};
-
-enum { kPhExpand = 0, kPhClaim, kPhOwn, kPhLabels, kPhExchange, kPhRedist, kPhWaitNarrow, kPhOther };
-
-// Shared memory of one engine CTA.
-struct EngineSmem {
-    EngineArgs args;
-    long long st[8];             // statistics (rcm_stats order), updated by thread 0
-    long long prof[8];           // per-phase ns (profile), updated by thread 0 of CTA 0
-    unsigned long long prof_t;   // timestamp of the last phase boundary
-    int scan[64];
-    int acc_cnt;                 // CTA count accumulator feeding the exchange
-    unsigned long long wkey[32]; // per-warp min keys of the last accumulate()
-    int ex[4];                   // exchange results: total, pre, maxcnt
-    unsigned long long ex_key;
-    int bc[8];
-    unsigned long long bck;
-    int tail;
-    int ntail[3];                // narrow levels-only loop: new-vertex counters, by level mod 3
-    struct {                     // state after a run of warp-0 levels, read by the whole CTA
-        int F, d, lstart, cb, lastF, bad, qb;
-        long long reached;
-        unsigned long long lk;
-    } wr;
-    int aflag;                   // async sweep: stop flag relayed to the CTA's warps
-    // middle tier: this CTA's part of each cluster exchange, read by the cluster's CTAs through
-    // distributed shared memory; double-buffered by epoch parity
-    unsigned long long xc_flag[2];  // (epoch << 32) | count, released at cluster scope
-    unsigned long long xc_key[2];   // min (degree, id) key of the CTA's slice
-    int cache[2][kCache];
-};
-
-enum { kStComponents = 0, kStSweeps, kStTraversals, kStLevels, kStMaxEcc, kStIsolated, kStNarrow, kStGrid };
 
 struct ExResult {
     int total;                // sum of the CTAs' counts
@@ -2006,6 +1912,50 @@ struct Engine {
         }
     }
 
+    // Whether this CTA's sweeps keep their state in shared memory (rcm_local.cuh): always where the
+    // rows are there too, otherwise for graphs that the kernel's bitmap holds.
+    __device__ bool local() const {
+        if constexpr (kSmem) return true;
+        if constexpr (kCtaOnly) return sm->loc.cap >= a->n;
+        return false;
+    }
+
+    // A levels-only / labelled sweep by the engine this graph runs on.
+    __device__ bool levels(int root, int& ecc, unsigned long long& last_key, long long& reached) {
+        if constexpr (kCtaOnly) {
+            if (local()) {
+                local_sweep<kSmem>(a, sm, 0, root, 0);
+                ecc = sm->wr.d;
+                last_key = sm->wr.lk;
+                reached = sm->wr.reached;
+                tick(kPhExpand);
+                stat_add(kStNarrow, ecc + 1);
+                return true;
+            }
+        }
+        if constexpr (!kSmem) return sweep_levels(root, ecc, last_key, reached);
+        return false;
+    }
+    __device__ bool labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size) {
+        if constexpr (kCtaOnly) {
+            if (local()) {
+                local_sweep<kSmem>(a, sm, 1, root, nv);
+                ecc = sm->wr.d;
+                last_key = sm->wr.lk;
+                size = (int)sm->wr.reached;
+                tick(kPhOwn);
+                stat_add(kStNarrow, ecc + 1);
+                if (sm->wr.bad) {
+                    fail(kErrInternal);
+                    return false;
+                }
+                return true;
+            }
+        }
+        if constexpr (!kSmem) return sweep_labelled(root, nv, ecc, last_key, size);
+        return false;
+    }
+
     // Degree-zero vertices are the first components in start-rule order: labels 0..Z-1 in
     // increasing id (an ordered compaction).
     __device__ bool label_isolated(int& Z) {
@@ -2050,6 +2000,15 @@ struct Engine {
         return barrier();
     }
 
+    // Claims of the vertices at labels [nv, nv + size) set as numbered (CTA engines).
+    __device__ void mark_numbered(int nv, int size) {
+        for (int i = threadIdx.x; i < size; i += blockDim.x) {
+            const int v = ldcg(a->perm + (a->n - 1 - (nv + i)));
+            if (in_graph(v)) *claim_p(v) = 0;
+        }
+        __syncthreads();
+    }
+
     // Start of the next component: min (degree, id) over the vertices not yet numbered.
     __device__ bool next_start(unsigned long long& out) {
         unsigned long long m = kKeyMax;
@@ -2087,12 +2046,12 @@ struct Engine {
             // last level as a levels-only one, and its level code is the faster of the two on the
             // whole grid. Its labels are discarded.
             int sz = 0;
-            if (!sweep_labelled(r, nv, ecc_prev, k1, sz)) return false;
+            if (!labelled(r, nv, ecc_prev, k1, sz)) return false;
             reached = sz;
             tick(kPhOther);
-            if (!reset_claims(nv, sz)) return false;
+            if (!local() && !reset_claims(nv, sz)) return false;
             tick(kPhOther);
-        } else if (!sweep_levels(r, ecc_prev, k1, reached)) {
+        } else if (!levels(r, ecc_prev, k1, reached)) {
             return false;
         }
         // The start vertex's component does not hold every vertex left: the others get a component
@@ -2101,7 +2060,7 @@ struct Engine {
         // it holds at least 3/4 of the vertices left (the rest, ordered concurrently afterwards,
         // costs less than the sweep would again): it takes the first labels either way. Otherwise
         // it is left to the table, to run beside the others, and its sweep is discarded.
-        const long long keep_min = !kCtaOnly ? (long long)a->cc_big : (kSmem ? 0 : (long long)kTinyMax + 1);
+        const long long keep_min = !kCtaOnly ? (long long)a->cc_big : (long long)kTinyMax + 1;
         if (all_left >= 0 && reached < all_left && reached < keep_min && 4 * reached < 3 * all_left) {
             size = -1;
             return true;
@@ -2116,7 +2075,7 @@ struct Engine {
             while (true) {
                 int ecc;
                 unsigned long long k2;
-                if (!sweep_labelled(r, nv, ecc, k2, size)) return false;
+                if (!labelled(r, nv, ecc, k2, size)) return false;
                 stat_add(kStSweeps, 1);
                 stat_add(kStTraversals, 1);
                 stat_add(kStLevels, ecc + 1);
@@ -2126,7 +2085,7 @@ struct Engine {
                 }
                 ecc_prev = ecc;
                 tick(kPhOther);
-                if (!reset_claims(nv, size)) return false;
+                if (!local() && !reset_claims(nv, size)) return false;
                 tick(kPhOther);
                 r = (int)(unsigned)(k2 & 0xffffffffu);
             }
@@ -2134,7 +2093,7 @@ struct Engine {
             while (true) {
                 int ecc;
                 unsigned long long k2;
-                if (!sweep_levels(r, ecc, k2, reached)) return false;
+                if (!levels(r, ecc, k2, reached)) return false;
                 stat_add(kStSweeps, 1);
                 stat_add(kStTraversals, 1);
                 stat_add(kStLevels, ecc + 1);
@@ -2143,7 +2102,7 @@ struct Engine {
                 r = (int)(unsigned)(k2 & 0xffffffffu);
             }
             unsigned long long k2;
-            if (!sweep_labelled(r, nv, ecc_root, k2, size)) return false;
+            if (!labelled(r, nv, ecc_root, k2, size)) return false;
             stat_add(kStTraversals, 1);
             stat_add(kStLevels, ecc_root + 1);
         }
@@ -2225,7 +2184,9 @@ struct Engine {
     // the status set.
     __device__ bool order_tiny(const int4& t, int* q, long long* st) {
         const int z = t.z, y = t.y;
-        int stamp = -1, reached = 0;
+        // (the shared-memory engine's stamps share their words with the labelled sweeps' claims, which
+        // are ~0 = -1 when unset and far below -2 otherwise)
+        int stamp = -2, reached = 0;
         unsigned long long k;
         int ecc_prev = tiny_bfs(t.x, stamp--, q, z, reached, k);
         if (ecc_prev < 0 || reached != z) {
@@ -2433,24 +2394,24 @@ struct Engine {
                 tried = true;
                 const int C = cc_prepare(nv, sm_sort, sm_sort_cap);
                 if (C == -2) return false;
+                // the table's sort may have used the local sweeps' memory
+                if (threadIdx.x == 0) sm->loc.gen = ~0u;
                 if (C > 0) {
-                    if constexpr (!kSmem) {
-                        // tiny components first, one per thread, all at once
-                        for (int i = threadIdx.x; i < C; i += blockDim.x) {
-                            const int4 t = a->cc_tab[i];
-                            if (t.z > kTinyMax) continue;
-                            if (!tab_ok(t, nv)) {
-                                fail_at(kSiteTable, i);
-                                break;
-                            }
-                            if (!order_tiny(t, a->qa + t.y, sm->st)) break;
+                    // tiny components first, one per thread, all at once
+                    for (int i = threadIdx.x; i < C; i += blockDim.x) {
+                        const int4 t = a->cc_tab[i];
+                        if (t.z > kTinyMax) continue;
+                        if (!tab_ok(t, nv)) {
+                            fail_at(kSiteTable, i);
+                            break;
                         }
-                        __syncthreads();
-                        if (ld_volatile(a->status) & (kErrInternal | kErrTimeout | kErrTooLarge)) return false;
+                        if (!order_tiny(t, a->qa + t.y, sm->st)) break;
                     }
+                    __syncthreads();
+                    if (ld_volatile(a->status) & (kErrInternal | kErrTimeout | kErrTooLarge)) return false;
                     for (int i = 0; i < C; ++i) {
                         const int4 t = a->cc_tab[i];
-                        if (!kSmem && t.z <= kTinyMax) continue;
+                        if (t.z <= kTinyMax) continue;
                         if (!tab_ok(t, nv)) {
                             fail_at(kSiteTable, i);
                             return false;
@@ -2478,6 +2439,8 @@ struct Engine {
             first = false;
             if (!component((int)(unsigned)(k0 & 0xffffffffu), nv, size, left)) return false;
             if (size < 0) continue;
+            // local sweeps leave no claims: the vertices just numbered are marked for the searches below
+            if (local() && nv + size < n) mark_numbered(nv, size);
             nv += size;
         }
         return true;

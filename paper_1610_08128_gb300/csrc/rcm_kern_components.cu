@@ -5,6 +5,6 @@
 
 namespace rcm {
 
-template __global__ void k_rcm_components<kComponentThreads>(EngineArgs);
+template __global__ void k_rcm_components<kComponentThreads>(EngineArgs, int, int, int);
 
 }  // namespace rcm

@@ -96,6 +96,12 @@ static const void* single_kernel(int threads, bool async = false, bool hybrid = 
     return (const void*)k_rcm_single<512, false, false>;
 }
 
+// k_rcm_components: hash slots and list entries of a component's local sweeps and the most dynamic
+// shared memory it may take (with its static part under the 227 KB of a CTA: graphs of up to 1.4M
+// vertices).
+constexpr int kComponentSlots = 2048;
+constexpr size_t kComponentSmem = 206 * 1024;
+
 constexpr int kSingleDynSmem = (int)((sizeof(unsigned long long) + sizeof(int)) * kCompSmem);
 
 static int single_blocks_per_sm(int threads, bool async = false, bool hybrid = false) {
@@ -109,6 +115,8 @@ static int single_blocks_per_sm(int threads, bool async = false, bool hybrid = f
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSingleDynSmem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, threads, kSingleDynSmem);
         g_single_blocks_per_sm[idx] = b;
+        cudaFuncSetAttribute((const void*)k_rcm_components<kComponentThreads>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kComponentSmem);
         cudaFuncSetAttribute(k_sort_rows_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(sizeof(unsigned long long) * kBigRowSmem));
     }
@@ -196,10 +204,10 @@ static const void* small_kernel(int threads) {
     return (const void*)k_rcm_small<512>;
 }
 
-// CTA width of the shared-memory executor when the caller does not choose one.
-// (256 was within a few percent of the best width on 2D and 3D grids and kNN meshes of 4,000
-// vertices on GB300; the best ranged from 128 on long 2D grids to 512 on many-component meshes.)
-static int small_default_threads(int) { return 256; }
+// CTA width of the shared-memory executor when the caller does not choose one: a level of up to 64
+// vertices is then one pass (the 64x64 grid 0.227 / 0.198 / 0.178 / 0.129 ms on 64 / 128 / 256 / 512
+// threads, a 1,000-point mesh of ten components 0.258 / 0.215 / 0.194 / 0.198 ms on GB300).
+static int small_default_threads(int) { return 512; }
 
 rcm_status single_launch(int n, long long nnz, const rcm_options& o, SingleLaunch* out) {
     const DeviceInfo& di = device_info();
@@ -401,9 +409,16 @@ static cudaError_t release_persisting(const char* win, size_t bytes, cudaStream_
 // kernel reads the table's size from the control block and exits at once when there is none.
 static cudaError_t launch_components(EngineArgs& args, const SingleLaunch& sl, cudaStream_t s) {
     const int blocks = std::max(1, sl.blocks * sl.threads / kComponentThreads);
-    void* cargs[] = {&args};
+    int cap = sl.cluster ? 0 : args.n, slots = kComponentSlots, entries = kComponentSlots;
+    size_t bytes = local_bytes(cap, slots, entries);
+    if (cap == 0 || bytes > kComponentSmem) {
+        cap = entries = 0;
+        slots = 1;
+        bytes = local_bytes(cap, slots, entries);
+    }
+    void* cargs[] = {&args, &cap, &slots, &entries};
     return cudaLaunchKernel((const void*)k_rcm_components<kComponentThreads>, dim3(blocks), dim3(kComponentThreads),
-                            cargs, 0, s);
+                            cargs, bytes, s);
 }
 
 cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* colidx, int* perm, char* base,

@@ -13,10 +13,12 @@ namespace rcm {
 // stamps and padded rows in shared memory (Engine<true, true>), so every level's row reads and
 // atomics stay inside one SM instead of going to L2.
 constexpr int kSmallMaxN = 4608;
-constexpr int kSmallSort = 256;  // component tables sorted in shared memory up to this size
+constexpr int kSmallList = 2048;  // list entries of its local sweeps
+constexpr int kSmallSort = kSmallList / 3;  // component tables sorted in shared memory up to this size
 
-// Shared-memory layout: claims (8n bytes) at 0, stamps (4n) and then the padded rows (32n, read
-// and written as 16-byte int4) each at the next 16-byte boundary.
+// Shared-memory layout: claims (8n bytes) at 0, stamps (4n; the labelled sweeps' claim words share
+// them) and then the padded rows (32n, read and written as 16-byte int4) each at the next 16-byte
+// boundary.
 inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 inline size_t small_vis_off(int n) { return align16(8 * (size_t)n); }
 inline size_t small_ell_off(int n) { return align16(small_vis_off(n) + 4 * (size_t)n); }
@@ -29,7 +31,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rcm_single(EngineArgs args, int
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads, 1) k_rcm_small(EngineArgs args, int vis_off, int ell_off);
 template <int kThreads>
-__global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args);
+__global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args, int local_cap, int local_slots, int local_entries);
 constexpr int kComponentThreads = 256;  // CTA width of k_rcm_components
 
 #ifndef RCM_KERNEL_DEFINITIONS
@@ -46,7 +48,7 @@ extern template __global__ void k_rcm_small<64>(EngineArgs, int, int);
 extern template __global__ void k_rcm_small<128>(EngineArgs, int, int);
 extern template __global__ void k_rcm_small<256>(EngineArgs, int, int);
 extern template __global__ void k_rcm_small<512>(EngineArgs, int, int);
-extern template __global__ void k_rcm_components<kComponentThreads>(EngineArgs);
+extern template __global__ void k_rcm_components<kComponentThreads>(EngineArgs, int, int, int);
 #else
 template <int kThreads, bool kAsync, bool kBottomUp>
 __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, EngineSmem& smem, int& s_item,
@@ -156,11 +158,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_rcm_single(EngineArgs args, int
 
 // The components that k_rcm_single's component table left to smaller engines: those of at most
 // kTinyMax vertices one per thread, the others (below the whole-grid size) one per CTA from a work
-// queue, with CTA barriers only and their levels of at most kWarpLevel vertices on warp 0. A kernel
-// of its own, so that neither its engine's code nor its CTA width weighs on the persistent grid
+// queue, with CTA barriers only. Their sweeps keep their state in shared memory (rcm_local.cuh) where
+// the whole graph's bitmap fits (local_cap >= n); otherwise in global memory, levels of at most
+// kWarpLevel vertices on warp 0. A kernel of its own, so that neither its engine's code nor its CTA width weighs on the persistent grid
 // kernel. Exits at once when the ordering built no table.
 template <int kThreads>
-__global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args) {
+__global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args, int local_cap, int local_slots, int local_entries) {
+    extern __shared__ __align__(16) unsigned s_local[];  // the local sweeps' state
     __shared__ EngineSmem smem;
     __shared__ int s_item;
     Ctl* ctl = args.ctl;
@@ -171,6 +175,7 @@ __global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args) {
     EngineArgs first = args;
     first.narrow_thr = 0x7fffffff;
     first.profile = 0;
+    if (threadIdx.x == 0) local_init(&smem.loc, local_cap, local_slots, local_entries, s_local);
     e.init(first, &smem);
     // visit stamps clear of the grid engine's (whose first sweep may have stamped a component)
     e.sweep_id = 1 << 24;
@@ -227,10 +232,16 @@ template <int kThreads>
 __global__ void __launch_bounds__(kThreads, 1) k_rcm_small(EngineArgs args, int vis_off, int ell_off) {
     extern __shared__ __align__(16) unsigned long long s_state[];
     __shared__ EngineSmem smem;
-    __shared__ unsigned long long s_sort[kSmallSort + kSmallSort / 2];
+    // the local sweeps' lists; component tables sort in the same bytes
+    __shared__ unsigned long long s_sort[kSmallList / 2];
+    unsigned* s_list = (unsigned*)s_sort;
+    __shared__ __align__(16) unsigned s_vis[kSmallMaxN / 32];
+    static_assert(kSmallMaxN % 128 == 0, "whole bitmap words");
     Ctl* ctl = args.ctl;
     if (ld_volatile(&ctl->status) & kErrBadCsr) return;
     const int n = args.n;
+    if (threadIdx.x == 0)
+        local_init(&smem.loc, kSmallMaxN, n, kSmallList, s_vis, (unsigned*)((char*)s_state + vis_off), nullptr, s_list);
     unsigned long long* claim = s_state;
     int* vis = (int*)((char*)s_state + vis_off);
     int4* ell = (int4*)((char*)s_state + ell_off);
