@@ -23,7 +23,7 @@ struct EngineArgs {
     int n;                       // vertices of this graph
     int v0;                      // global id of its first vertex (rows hold global ids)
     const int* rowptr;           // global rows (overflow neighbours of rows with degree > 7)
-    const int4* ell;             // 2 x int4 per vertex: 7 sorted neighbours (-1 padded) + degree
+    const int4* ell;             // 2 x int4 per vertex: 7 sorted neighbours (its own id where absent) + degree
     const int* adj;              // full sorted rows, valid for rows with degree > 7
     const int* deg;              // global
     unsigned long long* claim;   // global, 64-bit keys (kClaimNone = not reached)

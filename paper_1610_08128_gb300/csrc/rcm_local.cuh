@@ -39,7 +39,6 @@
 namespace rcm {
 
 constexpr int kLocalPasses = 4;    // passes of a wide level looked at together
-constexpr int kLocalBatch = 2;     // list batches of 32 looked at together
 constexpr int kLocalProbes = 64;   // table probes before a level is taken to be too wide for it
 // A list entry: (vertex, later its table slot) << kLocalPosBits | frontier position.
 constexpr int kLocalPosBits = 11;
@@ -48,8 +47,9 @@ static_assert(kCache <= 1 << kLocalPosBits, "positions of a level held in the sh
 constexpr int kLocalMax = 1 << (32 - kLocalPosBits);  // vertices of the largest graph
 constexpr int kLocalOverflow = 1 << 24;  // a warp's child count that says its level did not fit
 
-// Words of the bitmap of n vertices, in whole 16-byte groups.
-__host__ __device__ inline int local_vis_words(long long n) { return (int)((n + 127) / 128 * 4); }
+// Words of the bitmap of n vertices, in whole 16-byte groups. Bits follow the global ids (vertex w: bit
+// w mod 32 of word w / 32 - v0 / 32), so the first word may start in the middle.
+__host__ __device__ inline int local_vis_words(long long n) { return (int)((n + 31 + 127) / 128 * 4); }
 __host__ __device__ inline int local_id_bits(long long n) {
     int b = 1;
     while ((1LL << b) < n) ++b;
@@ -93,6 +93,11 @@ __device__ __forceinline__ int4 s_ld4(unsigned p) {
 __device__ __forceinline__ void s_st(unsigned p, unsigned v) {
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ unsigned s_or(unsigned p, unsigned v) {
+    unsigned old;
+    asm volatile("atom.shared.or.b32 %0, [%1], %2;" : "=r"(old) : "r"(p), "r"(v) : "memory");
+    return old;
+}
 __device__ __forceinline__ unsigned s_add(unsigned p, unsigned v) {
     unsigned old;
     asm volatile("atom.shared.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(p), "r"(v) : "memory");
@@ -110,26 +115,19 @@ __device__ __forceinline__ void s_red_or(unsigned p, unsigned v) {
     asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }
 
-// The same under a predicate, with no branch around it.
-__device__ __forceinline__ unsigned s_or_if(bool on, unsigned p, unsigned v, unsigned otherwise) {
+// Shared stores and atomics where a word is not zero / above a limit, predicated instead of branched around.
+__device__ __forceinline__ void s_st_nz(unsigned on, unsigned p, unsigned v) {
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; @q st.shared.u32 [%0], %1;}" ::"r"(p), "r"(v), "r"(on) : "memory");
+}
+__device__ __forceinline__ void s_red_min_nz(unsigned on, unsigned p, unsigned v) {
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; @q red.shared.min.u32 [%0], %1;}" ::"r"(p), "r"(v), "r"(on) : "memory");
+}
+// atom.cas where x > limit, else c.
+__device__ __forceinline__ unsigned s_cas_above(unsigned x, unsigned limit, unsigned p, unsigned c, unsigned v) {
     unsigned old;
-    asm volatile("{.reg .pred q; setp.ne.u32 q, %3, 0; mov.u32 %0, %4; @q atom.shared.or.b32 %0, [%1], %2;}"
-                 : "=&r"(old) : "r"(p), "r"(v), "r"((unsigned)on), "r"(otherwise) : "memory");
+    asm volatile("{.reg .pred q; setp.gt.u32 q, %4, %5; mov.u32 %0, %2; @q atom.shared.cas.b32 %0, [%1], %2, %3;}"
+                 : "=&r"(old) : "r"(p), "r"(c), "r"(v), "r"(x), "r"(limit) : "memory");
     return old;
-}
-__device__ __forceinline__ void s_st_if(bool on, unsigned p, unsigned v) {
-    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; @q st.shared.u32 [%0], %1;}"
-                 ::"r"(p), "r"(v), "r"((unsigned)on) : "memory");
-}
-__device__ __forceinline__ unsigned s_cas_if(bool on, unsigned p, unsigned c, unsigned v) {
-    unsigned old;
-    asm volatile("{.reg .pred q; setp.ne.u32 q, %4, 0; mov.u32 %0, %2; @q atom.shared.cas.b32 %0, [%1], %2, %3;}"
-                 : "=&r"(old) : "r"(p), "r"(c), "r"(v), "r"((unsigned)on) : "memory");
-    return old;
-}
-__device__ __forceinline__ void s_red_min_if(bool on, unsigned p, unsigned v) {
-    asm volatile("{.reg .pred q; setp.ne.u32 q, %2, 0; @q red.shared.min.u32 [%0], %1;}"
-                 ::"r"(p), "r"(v), "r"((unsigned)on) : "memory");
 }
 
 // The same with everything in one block of local_bytes(cap, slots, entries) bytes, 16-byte aligned.
@@ -175,7 +173,7 @@ struct Local {
         g = lane >> 3;
         k = lane & 7;
         below = (1u << lane) - 1u;
-        vis = s_addr(l.vis);
+        vis = s_addr(l.vis) - 4u * ((unsigned)v0 >> 5);
         hkey = s_addr(l.hkey);
         hval = s_addr(l.hval);
         srows = kDirect ? s_addr(rows) : 0u;
@@ -204,7 +202,11 @@ struct Local {
     __device__ void prefetch(int w) const {
         if constexpr (!kDirect) asm volatile("prefetch.global.L1 [%0];" ::"l"(rows + 8 * (size_t)w));
     }
-    __device__ bool visited(unsigned i) const { return (s_ld(vis + 4u * (i >> 5)) >> (i & 31)) & 1u; }
+    // The word of vertex w's bit, shifted so that the bit is the lowest.
+    __device__ unsigned visited_word(int w) const {
+        return __funnelshift_r(s_ld(vis + 4u * ((unsigned)w >> 5)), 0u, (unsigned)w);
+    }
+    __device__ bool visited(int w) const { return visited_word(w) & 1u; }
 
     // Vertices [j0, j1) of a level of F are this warp's: whole groups of 4, consecutive over the warps.
     __device__ void share(int F, int& j0, int& j1) const {
@@ -254,13 +256,15 @@ struct Local {
                 s_red_min(hval + 4 * s, value(j));
                 return (int)s;
             }
-            s = (s + 1) & (unsigned)(slots - 1);
+            s = next_slot(s, i);
         }
         return -1;
     }
+    // The probe after slot s: vertices that share a slot part ways.
+    __device__ unsigned next_slot(unsigned s, unsigned i) const { return (s + (i << 1) + 1u) & (unsigned)(slots - 1); }
 
-    // This lane's neighbour as a local id, out of range where it holds none (absent, or the degree).
-    __device__ unsigned neighbour(int x) const { return k < kEllNb ? (unsigned)(x - v0) : ~0u; }
+    // Rows hold only vertices of this graph (the validation pass saw to it), and absent neighbours are
+    // the vertex itself, which is always visited: nothing below checks a neighbour's range.
 
     // The row words of this lane for P passes of 4 vertices from position j (word 7: the degree).
     template <int P, class At>
@@ -297,11 +301,13 @@ struct Local {
         }
     }
 
-    // Entry r of this warp's list: vertex and position.
-    __device__ void put(bool on, int r, unsigned i, int j) const {
-        s_st_if(on, list + 4 * r, i << kLocalPosBits | (unsigned)j);
-        if constexpr (kDirect) s_red_min_if(on, hval + 4 * i, value(j));
+    // List entry at shared address p, where `on` is not zero: vertex w with frontier position j,
+    // jbase = j - (v0 << kLocalPosBits).
+    __device__ void put(unsigned on, unsigned p, int w, unsigned jbase) const {
+        s_st_nz(on, p, ((unsigned)w << kLocalPosBits) + jbase);
+        if constexpr (kDirect) s_red_min_nz(on, hval + 4 * (unsigned)(w - v0), value0 | (jbase & kLocalPos));
     }
+    __device__ unsigned list_base(int j) const { return (unsigned)j - ((unsigned)v0 << kLocalPosBits); }
 
     // The padded row of vertex u.
     __device__ void row(int u, int (&r)[8]) const {
@@ -331,52 +337,64 @@ struct Local {
     // warp's list in (position, row) order; count goes past qcap without writing.
     __device__ void collect(unsigned cache, int jb, int j1, int& count) {
         const int j = jb + lane;
-        const bool on = j < j1;
+        const unsigned on = j < j1 ? 1u : 0u;
         int r[8];
         row((int)s_ld(cache + 4 * min(j, j1 - 1)), r);
-        unsigned mask = 0;
+        unsigned open[kEllNb];
+        int c = 0;
 #pragma unroll
-        for (int q = 0; q < kEllNb; ++q) {
-            const unsigned i = (unsigned)(r[q] - v0);
-            const bool ok = i < (unsigned)n;
-            mask |= (ok && !visited(ok ? i : 0u) ? 1u : 0u) << q;
+        for (int q = 0; q < 4; ++q) open[q] = ~visited_word(r[q]) & on;
+#pragma unroll
+        for (int q = 4; q < kEllNb; ++q) open[q] = 0;
+        const bool wide = __any_sync(0xffffffffu, r[7] > 4);  // the row's second half is in use
+        if (wide) {
+#pragma unroll
+            for (int q = 4; q < kEllNb; ++q) open[q] = ~visited_word(r[q]) & on;
         }
-        if (!on) mask = 0;
-        const unsigned lm = __ballot_sync(0xffffffffu, on && r[7] > kEllNb);
-        int c = __popc(mask), total, at;
+#pragma unroll
+        for (int q = 0; q < kEllNb; ++q) c += (int)open[q];
+        const unsigned lm = wide ? __ballot_sync(0xffffffffu, on && r[7] > kEllNb) : 0u;
+        int total, at;
         if (!lm) {
-            at = count + prefix7(c, total);
+            at = prefix7(c, total);
         } else {
             // rows with more than 7 entries: the rest is counted by the whole warp first
-            long_list(cache, jb, r[7], lm, [&](int src, unsigned, bool open) {
-                const int m = __popc(__ballot_sync(0xffffffffu, open));
+            long_list(cache, jb, r[7], lm, [&](int src, int, bool o) {
+                const int m = __popc(__ballot_sync(0xffffffffu, o));
                 if (lane == src) c += m;
             });
             const int incl = warp_incl_scan(c);
             total = __shfl_sync(0xffffffffu, incl, 31);
-            at = count + incl - c;
+            at = incl - c;
         }
+        unsigned p = list + 4u * (unsigned)(count + at);
         count += total;
         if (count > qcap) return;  // the caller sees the overflow
+        const unsigned jbase = list_base(j);
 #pragma unroll
-        for (int q = 0; q < kEllNb; ++q) {
-            const bool open = (mask >> q) & 1u;
-            put(open, at, (unsigned)(r[q] - v0), j);
-            at += open ? 1 : 0;
+        for (int q = 0; q < 4; ++q) {
+            put(open[q], p, r[q], jbase);
+            p += 4u * open[q];
+        }
+        if (wide) {
+#pragma unroll
+            for (int q = 4; q < kEllNb; ++q) {
+                put(open[q], p, r[q], jbase);
+                p += 4u * open[q];
+            }
         }
         if (lm) {
-            long_list(cache, jb, r[7], lm, [&](int src, unsigned i, bool open) {
-                const unsigned m = __ballot_sync(0xffffffffu, open);
-                const int base = __shfl_sync(0xffffffffu, at, src);
-                put(open, base + __popc(m & below), i, jb + src);
-                if (lane == src) at += __popc(m);
+            long_list(cache, jb, r[7], lm, [&](int src, int w, bool o) {
+                const unsigned m = __ballot_sync(0xffffffffu, o);
+                const unsigned base = __shfl_sync(0xffffffffu, p, src);
+                put(o ? 1u : 0u, base + 4u * (unsigned)__popc(m & below), w, list_base(jb + src));
+                if (lane == src) p += 4u * (unsigned)__popc(m);
             });
         }
     }
 
-    // fn(src, i, open) for the entries beyond the padded rows of the lanes lm (vertex jb + src, degree
-    // dg on its lane), 32 at a time by the whole warp: the entry as a local id and whether it is an
-    // unvisited vertex.
+    // fn(src, w, open) for the entries beyond the padded rows of the lanes lm (vertex jb + src, degree
+    // dg on its lane), 32 at a time by the whole warp: the entry and whether it is an unvisited vertex.
     template <class Fn>
     __device__ void long_list(unsigned cache, int jb, int dg, unsigned lm, Fn fn) const {
         for (unsigned m = lm; m; m &= m - 1) {
@@ -390,76 +408,47 @@ struct Local {
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     if (e0 + 32 * t >= d) break;
-                    const unsigned i = (unsigned)(w[t] - v0);
-                    const bool ok = w[t] >= 0 && i < (unsigned)n;
-                    fn(src, i, ok && !visited(ok ? i : 0u));
+                    fn(src, w[t], w[t] >= 0 && !visited(max(w[t], v0)));
                 }
             }
         }
     }
 
-    // Entries [b, b + 32 Q) of this warp's list (of c) claim their vertices in the table, and keep the slot.
-    // The first probes run side by side; what they do not settle goes on one by one. False where the
-    // table is too full.
-    template <int Q>
+    // Entries [b, b + 32) of this warp's list (of c) claim their vertices in the table, and keep the slot.
+    // The first probe is straight-line; what it does not settle goes on in a loop. False where the table
+    // is too full.
     __device__ bool claim_list(int b, int c) const {
-        unsigned e[Q], s[Q], cur[Q];
-        bool on[Q], left = false, ok = true;
-#pragma unroll
-        for (int p = 0; p < Q; ++p) {
-            on[p] = b + 32 * p + lane < c;
-            e[p] = s_ld(list + 4 * min(b + 32 * p + lane, c - 1));
+        const unsigned ids = (1u << idbits) - 1u;
+        const unsigned on = b + lane < c ? 1u : 0u;
+        const unsigned e = s_ld(list + 4 * min(b + lane, c - 1));
+        const unsigned i = e >> kLocalPosBits;
+        unsigned s = (i * 0x9E3779B1u) >> shift;
+        const unsigned cur = s_ld(hkey + 4 * s);
+        // x: the slot's word without the generation's part, above ids where it is of an earlier generation
+        // (empty); lanes past the end see no empty slot
+        const unsigned x = on ? cur ^ word0 : 0u;
+        const unsigned old = s_cas_above(x, ids, hkey + 4 * s, cur, word0 | i) ^ word0;
+        const bool made = x > ids && old == x;
+        if (made) prefetch(v0 + (int)i);  // a vertex of the next level
+        const unsigned hit = made || old == i ? on : 0u;
+        s_red_min_nz(hit, hval + 4 * s, value0 | (e & kLocalPos));
+        bool ok = true;
+        if (hit != on) {
+            const int t = claim_slot(i, (int)(e & kLocalPos), next_slot(s, i));
+            ok = t >= 0;
+            s = ok ? (unsigned)t : 0u;  // (any slot: the level is run again)
         }
-#pragma unroll
-        for (int p = 0; p < Q; ++p) {
-            s[p] = ((e[p] >> kLocalPosBits) * 0x9E3779B1u) >> shift;
-            cur[p] = s_ld(hkey + 4 * s[p]);
-        }
-#pragma unroll
-        for (int p = 0; p < Q; ++p) {
-            const unsigned i = e[p] >> kLocalPosBits, word = word0 | i;
-            const bool empty = on[p] && (cur[p] >> idbits) != gen;  // an entry of an earlier generation
-            const unsigned old = s_cas_if(empty, hkey + 4 * s[p], cur[p], word);
-            if (empty && old == cur[p]) prefetch(v0 + (int)i);  // a vertex of the next level
-            const bool hit = on[p] && ((empty && old == cur[p]) || old == word);
-            s_red_min_if(hit, hval + 4 * s[p], value((int)(e[p] & kLocalPos)));
-            on[p] = on[p] && !hit;
-            left |= on[p];
-        }
-        if (left) {
-#pragma unroll
-            for (int p = 0; p < Q; ++p) {
-                if (!on[p]) continue;
-                const int t = claim_slot(e[p] >> kLocalPosBits, (int)(e[p] & kLocalPos), (s[p] + 1) & (unsigned)(slots - 1));
-                ok &= t >= 0;
-                s[p] = t >= 0 ? (unsigned)t : 0u;  // (any slot: the level is run again)
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < Q; ++p)
-            s_st_if(b + 32 * p + lane < c, list + 4 * (b + 32 * p + lane), s[p] << kLocalPosBits | (e[p] & kLocalPos));
+        s_st_nz(on, list + 4 * (b + lane), s << kLocalPosBits | (e & kLocalPos));
         return ok;
     }
 
-    // Which of the entries [b, b + 32 Q) hold a child of their position, as ballots, and their vertices
-    // or slots; returns the number of children.
-    template <int Q>
-    __device__ int owned_list(int b, int c, unsigned (&own)[Q], unsigned (&at)[Q]) const {
-        unsigned e[Q], v[Q];
-#pragma unroll
-        for (int p = 0; p < Q; ++p) e[p] = s_ld(list + 4 * min(b + 32 * p + lane, c - 1));
-#pragma unroll
-        for (int p = 0; p < Q; ++p) {
-            at[p] = e[p] >> kLocalPosBits;
-            v[p] = s_ld(hval + 4 * at[p]);
-        }
-        int count = 0;
-#pragma unroll
-        for (int p = 0; p < Q; ++p) {
-            own[p] = __ballot_sync(0xffffffffu, b + 32 * p + lane < c && v[p] == value((int)(e[p] & kLocalPos)));
-            count += __popc(own[p]);
-        }
-        return count;
+    // Which of the entries [b, b + 32) hold a child of their position, as a ballot, and what this lane's
+    // names (its slot of the table, direct claims: its vertex).
+    __device__ unsigned owned_list(int b, int c, unsigned& at) const {
+        const unsigned e = s_ld(list + 4 * min(b + lane, c - 1));
+        at = e >> kLocalPosBits;
+        const unsigned v = s_ld(hval + 4 * at);
+        return __ballot_sync(0xffffffffu, b + lane < c && v == (value0 | (e & kLocalPos)));
     }
 
     // The rank of this warp's first child among the level's, from the warps' counts; kids: their sum.
@@ -472,12 +461,11 @@ struct Local {
         return __reduce_add_sync(0xffffffffu, lane < wid ? c : 0);
     }
 
-    // Child r of the level at labels lab0..: vertex v0 + i.
-    __device__ void emit(unsigned i, int r, int lab0, unsigned next) {
-        const int w = v0 + (int)i;
+    // Child r of the level at labels lab0..: vertex w.
+    __device__ void emit(int w, int r, int lab0, unsigned next) {
         if (r < kCache) s_st(next + 4 * r, (unsigned)w);
         perm_end[-(lab0 + r)] = w;
-        s_red_or(vis + 4 * (i >> 5), 1u << (i & 31));
+        s_red_or(vis + 4u * ((unsigned)w >> 5), 1u << ((unsigned)w & 31u));
     }
 
     // One labelled level of F vertices at labels [lstart, lstart + F), positions below kCache in `cache`:
@@ -490,21 +478,22 @@ struct Local {
         // A warp with one pass of padded rows needs no list: each lane keeps its neighbour.
         bool held = j1 - jb <= 4;
         bool open = false, fits = true;
-        unsigned i0 = 0, s0 = 0;
+        int x = 0;
+        unsigned s0 = 0;
         int c = 0;
         if (held && jb < j1) {
-            const int x = row_word((int)s_ld(cache + 4 * min(jb + g, j1 - 1)));
+            x = row_word((int)s_ld(cache + 4 * min(jb + g, j1 - 1)));
             const bool on = jb + g < j1;
-            i0 = (unsigned)(x - v0);
-            const bool ok = on && k < kEllNb && i0 < (unsigned)n;
-            open = ok && !visited(ok ? i0 : 0u);
-            held = !__any_sync(0xffffffffu, on && k == 7 && x > kEllNb);
-            if (held) {
+            held = !__any_sync(0xffffffffu, k == 7 && x > kEllNb);
+            const unsigned seen = visited_word(k < kEllNb ? x : v0);
+            open = on && k < kEllNb && held && !(seen & 1u);
+            if (open) {
+                const unsigned i = (unsigned)(x - v0);
                 if constexpr (kDirect) {
-                    s_red_min_if(open, hval + 4 * i0, value(jb + g));
-                    s0 = i0;
-                } else if (open) {
-                    const int s = claim_slot(i0, jb + g, (i0 * 0x9E3779B1u) >> shift);
+                    s_red_min(hval + 4 * i, value(jb + g));
+                    s0 = i;
+                } else {
+                    const int s = claim_slot(i, jb + g, (i * 0x9E3779B1u) >> shift);
                     fits = s >= 0;
                     s0 = fits ? (unsigned)s : 0u;
                 }
@@ -517,20 +506,22 @@ struct Local {
             if (c > qcap) c = 0;
             __syncwarp();
             if constexpr (!kDirect) {
-                for (int b = 0; b < c; b += 32 * kLocalBatch) fits &= claim_list<kLocalBatch>(b, c);
+                for (int b = 0; b < c; b += 32) fits &= claim_list(b, c);
             }
         }
         fits = __all_sync(0xffffffffu, fits);
         __syncthreads();
-        // a vertex's children are the neighbours whose smallest claim is its position; the first
-        // batches' stay in registers
-        unsigned own[kLocalBatch], id[kLocalBatch];
+        // a vertex's children are the neighbours whose smallest claim is its position
+        unsigned own = 0, id = 0;
         int count = 0;
         if (held) {
-            own[0] = __ballot_sync(0xffffffffu, open && s_ld(hval + 4 * s0) == value(jh));
-            count = __popc(own[0]);
+            own = __ballot_sync(0xffffffffu, open && s_ld(hval + 4 * s0) == value(jh));
+            count = __popc(own);
         } else {
-            for (int b = 0; b < c; b += 32 * kLocalBatch) count += owned_list<kLocalBatch>(b, c, own, id);
+            for (int b = 0; b < c; b += 32) {
+                own = owned_list(b, c, id);
+                count += __popc(own);
+            }
         }
         int kids;
         int rank = rank_warps(fits ? count : kLocalOverflow, kids);
@@ -541,18 +532,15 @@ struct Local {
             return 0;
         }
         if (held) {
-            if ((own[0] >> lane) & 1u) emit(i0, rank + __popc(own[0] & below), lab0, next);
+            if ((own >> lane) & 1u) emit(x, rank + __popc(own & below), lab0, next);
         } else {
-            for (int b = 0; b < c; b += 32 * kLocalBatch) {
-                if (c > 32 * kLocalBatch) owned_list<kLocalBatch>(b, c, own, id);
-#pragma unroll
-                for (int p = 0; p < kLocalBatch; ++p) {
-                    if ((own[p] >> lane) & 1u) {
-                        const unsigned i = kDirect ? id[p] : s_ld(hkey + 4 * id[p]) & ((1u << idbits) - 1u);
-                        emit(i, rank + __popc(own[p] & below), lab0, next);
-                    }
-                    rank += __popc(own[p]);
+            for (int b = 0; b < c; b += 32) {
+                if (c > 32) own = owned_list(b, c, id);
+                if ((own >> lane) & 1u) {
+                    const unsigned i = kDirect ? id : s_ld(hkey + 4 * id) & ((1u << idbits) - 1u);
+                    emit(v0 + (int)i, rank + __popc(own & below), lab0, next);
                 }
+                rank += __popc(own);
             }
         }
         __syncthreads();
@@ -567,24 +555,25 @@ struct Local {
         share(F, j0, j1);
         auto at = [&](int j) { return labelled_at(j, cache, lstart); };
         constexpr int P = kLocalPasses;
-        auto open = [&](unsigned i) { return i < (unsigned)n && !visited(i); };
-        auto lower = [&](unsigned i, int j) {
-            if constexpr (kDirect) s_red_min(hval + 4 * i, value(j));
-            else atomicMin(a->claim + v0 + i, global_key(j));
+        // no vertex: below v0 (this lane has no neighbour)
+        auto open = [&](int w) { return w >= v0 && !visited(w); };
+        auto lower = [&](int w, int j) {
+            if constexpr (kDirect) s_red_min(hval + 4 * (unsigned)(w - v0), value(j));
+            else atomicMin(a->claim + w, global_key(j));
         };
-        auto mine = [&](unsigned i, int j) {
-            if constexpr (kDirect) return open(i) && s_ld(hval + 4 * i) == value(j);
-            else return open(i) && __ldcg(a->claim + v0 + i) == global_key(j);
+        auto mine = [&](int w, int j) {
+            if constexpr (kDirect) return open(w) && s_ld(hval + 4 * (unsigned)(w - v0)) == value(j);
+            else return open(w) && __ldcg(a->claim + w) == global_key(j);
         };
+        auto neighbour = [&](int y) { return k < kEllNb ? y : -1; };
         int x[P];
         for (int jb = j0; jb < j1; jb += 4 * P) {
             load(at, jb + g, j1, x);
 #pragma unroll
             for (int p = 0; p < P; ++p) {
-                const unsigned i = neighbour(x[p]);
-                if (open(i)) lower(i, jb + g + 4 * p);
+                if (open(neighbour(x[p]))) lower(x[p], jb + g + 4 * p);
                 long_rows(at, jb + 4 * p, x[p], __ballot_sync(0xffffffffu, k == 7 && x[p] > kEllNb), [&](int j, int w) {
-                    if (w >= 0 && open((unsigned)(w - v0))) lower((unsigned)(w - v0), j);
+                    if (open(w)) lower(w, j);
                 });
             }
         }
@@ -605,7 +594,7 @@ struct Local {
             for (int p = 0; p < P; ++p) {
                 count += __popc(own[p]);
                 long_rows(at, jb + 4 * p, x[p], __ballot_sync(0xffffffffu, k == 7 && x[p] > kEllNb), [&](int j, int w) {
-                    count += __popc(__ballot_sync(0xffffffffu, w >= 0 && mine((unsigned)(w - v0), j)));
+                    count += __popc(__ballot_sync(0xffffffffu, mine(w, j)));
                 });
             }
         }
@@ -613,8 +602,8 @@ struct Local {
         int rank = rank_warps(count, kids);
         const int lab0 = lstart + F;
         if (lab0 + kids > n) return -1;
-        auto put = [&](unsigned m, unsigned i) {
-            if ((m >> lane) & 1u) emit(i, rank + __popc(m & below), lab0, next);
+        auto put = [&](unsigned m, int w) {
+            if ((m >> lane) & 1u) emit(w, rank + __popc(m & below), lab0, next);
             rank += __popc(m);
         };
         for (int jb = j0; jb < j1; jb += 4 * P) {
@@ -624,11 +613,10 @@ struct Local {
                 const unsigned lm = __ballot_sync(0xffffffffu, k == 7 && x[p] > kEllNb);
                 for (int v = 0; v < 4; ++v) {
                     const unsigned of = lm ? 0xffu << (8 * v) : 0xffffffffu;
-                    put(own[p] & of, neighbour(x[p]));
+                    put(own[p] & of, x[p]);
                     if (!lm) break;
                     long_rows(at, jb + 4 * p, x[p], lm & of, [&](int j, int w) {
-                        const unsigned i = (unsigned)(w - v0);
-                        put(__ballot_sync(0xffffffffu, w >= 0 && mine(i, j)), i);
+                        put(__ballot_sync(0xffffffffu, mine(w, j)), w);
                     });
                 }
             }
@@ -656,23 +644,29 @@ struct Local {
             if (lane == 0 && count) r = (int)s_add(tail, (unsigned)count);
             return __shfl_sync(0xffffffffu, r, 0);
         };
-        auto reach = [&](unsigned i) {
-            const bool ok = i < (unsigned)n;
-            return !((s_or_if(ok, vis + 4 * (i >> 5), 1u << (i & 31), ~0u) >> (i & 31)) & 1u);
+        // 1 where vertex w was not visited; it is now
+        auto reach = [&](int w) {
+            const unsigned bit = 1u << ((unsigned)w & 31u);
+            return s_or(vis + 4u * ((unsigned)w >> 5), bit) & bit ? 0u : 1u;
+        };
+        auto rest = [&](int u, int d) {  // the entries of a long row beyond the padded ones, by the warp
+            const int* rw = a->adj + __ldg(a->rowptr + u);
+            for (int e = kEllNb; e < d; e += 32) {
+                const int w = e + lane < d ? __ldg(rw + e + lane) : -1;
+                const unsigned f = __ballot_sync(0xffffffffu, w >= 0 && reach(w));
+                put(f, w, reserve(__popc(f)));
+            }
         };
         if (j1 - jb <= 4) {
             // one pass, eight lanes per vertex
             if (jb >= j1) return;
             const bool on = jb + g < j1;
-            const int x = row_word(at(min(jb + g, j1 - 1)));
-            const unsigned m = __ballot_sync(0xffffffffu, reach(on && k < kEllNb ? (unsigned)(x - v0) : ~0u));
+            const int u = at(min(jb + g, j1 - 1));
+            const int x = row_word(u);
+            const unsigned m = __ballot_sync(0xffffffffu, on && k < kEllNb && reach(x));
             put(m, x, reserve(__popc(m)));
-            const unsigned lm = __ballot_sync(0xffffffffu, on && k == 7 && x > kEllNb);
-            if (lm)
-                long_rows(at, jb, x, lm, [&](int, int w) {
-                    const unsigned f = __ballot_sync(0xffffffffu, reach(w >= 0 ? (unsigned)(w - v0) : ~0u));
-                    put(f, w, reserve(__popc(f)));
-                });
+            for (unsigned lm = __ballot_sync(0xffffffffu, on && k == 7 && x > kEllNb); lm; lm &= lm - 1)
+                rest(__shfl_sync(0xffffffffu, u, __ffs(lm) - 1), __shfl_sync(0xffffffffu, x, __ffs(lm) - 1));
             return;
         }
         for (; jb < j1; jb += 32) {
@@ -681,40 +675,43 @@ struct Local {
             const int u = at(min(jb + lane, j1 - 1));
             int r[8];
             row(u, r);
-            unsigned mask = 0;
+            unsigned fresh[kEllNb];
 #pragma unroll
-            for (int q = 0; q < kEllNb; ++q) mask |= (reach(on ? (unsigned)(r[q] - v0) : ~0u) ? 1u : 0u) << q;
-            int total;
-            int pos = prefix7(__popc(mask), total);
+            for (int q = 0; q < kEllNb; ++q) fresh[q] = 0;
+            const bool wide = __any_sync(0xffffffffu, r[7] > 4);  // the row's second half is in use
+            if (on) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) fresh[q] = reach(r[q]);
+                if (wide) {
+#pragma unroll
+                    for (int q = 4; q < kEllNb; ++q) fresh[q] = reach(r[q]);
+                }
+            }
+            int c = 0, total;
+#pragma unroll
+            for (int q = 0; q < kEllNb; ++q) c += (int)fresh[q];
+            int pos = prefix7(c, total);
             pos += reserve(total);
 #pragma unroll
             for (int q = 0; q < kEllNb; ++q)
-                if ((mask >> q) & 1u) {
+                if (fresh[q]) {
                     prefetch(r[q]);
                     if (pos < kCache) s_st(next + 4 * pos, (unsigned)r[q]); else nxt[pos] = r[q];
                     ++pos;
                 }
-            for (unsigned lm = __ballot_sync(0xffffffffu, on && r[7] > kEllNb); lm; lm &= lm - 1) {
-                const int src = __ffs(lm) - 1;
-                const int d = __shfl_sync(0xffffffffu, r[7], src);
-                const int* rw = a->adj + __ldg(a->rowptr + __shfl_sync(0xffffffffu, u, src));
-                for (int e = kEllNb; e < d; e += 32) {
-                    const int w = e + lane < d ? __ldg(rw + e + lane) : -1;
-                    const unsigned f = __ballot_sync(0xffffffffu, reach(w >= 0 ? (unsigned)(w - v0) : ~0u));
-                    put(f, w, reserve(__popc(f)));
-                }
-            }
+            if (!wide) continue;
+            for (unsigned lm = __ballot_sync(0xffffffffu, on && r[7] > kEllNb); lm; lm &= lm - 1)
+                rest(__shfl_sync(0xffffffffu, u, __ffs(lm) - 1), __shfl_sync(0xffffffffu, r[7], __ffs(lm) - 1));
         }
     }
 
     // Visited bits cleared, the root's set; the caller's next barrier orders them.
     __device__ void start(int root) {
         uint4* v = (uint4*)sm->loc.vis;
-        for (int i = threadIdx.x; i < (n + 127) / 128; i += blockDim.x) v[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (int i = threadIdx.x; i < local_vis_words(n) / 4; i += blockDim.x) v[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
         if (threadIdx.x == 0) {
-            const unsigned i = (unsigned)(root - v0);
-            sm->loc.vis[i >> 5] |= 1u << (i & 31);
+            sm->loc.vis[((unsigned)root >> 5) - ((unsigned)v0 >> 5)] |= 1u << ((unsigned)root & 31u);
             sm->cache[0][0] = root;
         }
     }

@@ -99,7 +99,7 @@ __device__ __forceinline__ void write_sorted_row(int v, int a, int m, const unsi
     for (int i = t; i < m; i += nt) adj[a + i] = (int)(unsigned)(keys[i] & 0xffffffffu);
     if (t == 0) {
         int r[8];
-        for (int i = 0; i < 7; ++i) r[i] = i < m ? (int)(unsigned)(keys[i] & 0xffffffffu) : -1;
+        for (int i = 0; i < 7; ++i) r[i] = i < m ? (int)(unsigned)(keys[i] & 0xffffffffu) : v;
         r[7] = m;
         store_ell(ell, v, r);
     }

@@ -10,8 +10,8 @@ constexpr int kBigRowSmem = 8192;    // rows sorted in shared memory by one CTA 
 constexpr int kBigRowThreads = 256;  // CTA width of k_sort_rows_big: 8 warps
 constexpr int kWarpRowMax = kBigRowSmem / (kBigRowThreads / 32);  // rows sorted by one warp (its 8 KB slice)
 
-// Padded row of vertex v: its first 7 neighbours in (degree, id) order (-1 where absent) and its
-// degree in slot 7, as two 16-byte stores (one 32-byte sector per vertex).
+// Padded row of vertex v: its first 7 neighbours in (degree, id) order (v itself where absent: readers
+// that look at all 7 find a vertex that is already visited) and its degree in slot 7, as two 16-byte stores (one 32-byte sector per vertex).
 __device__ __forceinline__ void store_ell(int4* ell, int v, const int (&r)[8]) {
     ell[2 * (size_t)v] = make_int4(r[0], r[1], r[2], r[3]);
     ell[2 * (size_t)v + 1] = make_int4(r[4], r[5], r[6], r[7]);
@@ -114,7 +114,7 @@ __device__ __forceinline__ void sort_row8(int v, int a, int len, const int* __re
     cmp_swap(k[1], k[2]); cmp_swap(k[3], k[4]); cmp_swap(k[5], k[6]);
     int r[8];
 #pragma unroll
-    for (int i = 0; i < 7; ++i) r[i] = i < m ? (int)(unsigned)(k[i] & 0xffffffffu) : -1;
+    for (int i = 0; i < 7; ++i) r[i] = i < m ? (int)(unsigned)(k[i] & 0xffffffffu) : v;
     r[7] = m;
     store_ell(ell, v, r);
     if (m > 7) {
@@ -148,7 +148,7 @@ __device__ __forceinline__ void sort_small_row(int v, const int* __restrict__ ro
     }
     int r[8];
 #pragma unroll
-    for (int i = 0; i < 7; ++i) r[i] = i < m ? (int)(unsigned)(key[i] & 0xffffffffu) : -1;
+    for (int i = 0; i < 7; ++i) r[i] = i < m ? (int)(unsigned)(key[i] & 0xffffffffu) : v;
     r[7] = m;
     store_ell(ell, v, r);
     if (m > 7)

@@ -96,10 +96,11 @@ static const void* single_kernel(int threads, bool async = false, bool hybrid = 
     return (const void*)k_rcm_single<512, false, false>;
 }
 
-// k_rcm_components: hash slots and list entries of a component's local sweeps and the most dynamic
+// k_rcm_components: the most hash slots, the list entries of a component's local sweeps and the most dynamic
 // shared memory it may take (with its static part under the 227 KB of a CTA: graphs of up to 1.4M
 // vertices).
-constexpr int kComponentSlots = 2048;
+constexpr int kComponentSlots = 8192;
+constexpr int kComponentEntries = 3072;
 constexpr size_t kComponentSmem = 206 * 1024;
 
 constexpr int kSingleDynSmem = (int)((sizeof(unsigned long long) + sizeof(int)) * kCompSmem);
@@ -409,7 +410,8 @@ static cudaError_t release_persisting(const char* win, size_t bytes, cudaStream_
 // kernel reads the table's size from the control block and exits at once when there is none.
 static cudaError_t launch_components(EngineArgs& args, const SingleLaunch& sl, cudaStream_t s) {
     const int blocks = std::max(1, sl.blocks * sl.threads / kComponentThreads);
-    int cap = sl.cluster ? 0 : args.n, slots = kComponentSlots, entries = kComponentSlots;
+    int cap = sl.cluster ? 0 : args.n, slots = kComponentSlots, entries = kComponentEntries;
+    while (slots > 2048 && local_bytes(cap, slots, entries) > kComponentSmem) slots /= 2;
     size_t bytes = local_bytes(cap, slots, entries);
     if (cap == 0 || bytes > kComponentSmem) {
         cap = entries = 0;

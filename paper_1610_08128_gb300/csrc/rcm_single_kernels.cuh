@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rcm_small(EngineArgs args, int 
     // the local sweeps' lists; component tables sort in the same bytes
     __shared__ unsigned long long s_sort[kSmallList / 2];
     unsigned* s_list = (unsigned*)s_sort;
-    __shared__ __align__(16) unsigned s_vis[kSmallMaxN / 32];
+    __shared__ __align__(16) unsigned s_vis[kSmallMaxN / 32 + 4];  // local_vis_words(kSmallMaxN)
     static_assert(kSmallMaxN % 128 == 0, "whole bitmap words");
     Ctl* ctl = args.ctl;
     if (ld_volatile(&ctl->status) & kErrBadCsr) return;
