@@ -127,6 +127,8 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks<kThreads>()) k_rcm_
         a.aq_cap = 0;
         a.mid_k = 0;  // CTA engines: no middle tier
         a.mid_thr = 0;
+        a.local_hi = a.local_slots = a.local_entries = 0;  // (the grid executor's)
+        a.gvis = nullptr;
         __syncthreads();
         e.init(a, &smem);
         e.sm_sort = (unsigned long long*)s_local;

@@ -82,6 +82,17 @@ template <bool kCtaOnly, bool kSmem, bool kAsync, bool kBottomUp, bool kWarp>
 __device__ __noinline__ void run_warp_labelled(const EngineArgs* a, EngineSmem* sm, int d, int lstart, int F, int cb,
                                                const int* sh, const int* g, int step);
 
+// The whole grid's sweeps and, inside the labelled one, its runs of whole-grid levels, out of line: one
+// copy each, with registers of its own (inlined into one kernel they spill: 192^3 grid 7.1 against 6.8
+// ms). Results in sm->sw and sm->wr.
+template <bool kAsync, bool kBottomUp>
+__device__ __noinline__ bool run_grid_levels_only(const EngineArgs* a, EngineSmem* sm, int root);
+template <bool kAsync, bool kBottomUp>
+__device__ __noinline__ bool run_grid_labelled(const EngineArgs* a, EngineSmem* sm, int root, int nv);
+template <bool kAsync, bool kBottomUp>
+__device__ __noinline__ bool run_grid_levels(const EngineArgs* a, EngineSmem* sm, int d, int lstart, int nv,
+                                             const int* g, int cnt, int prev_start, int prev_size);
+
 template <bool kCtaOnly, bool kSmem = false, bool kAsync = false, bool kBottomUp = false, bool kWarp = kSmem>
 struct Engine {
     static_assert(kCtaOnly || !kSmem, "shared-memory state needs a CTA engine");
@@ -372,6 +383,85 @@ struct Engine {
     __device__ bool barrier() {
         ExResult r;
         return exchange(r, false);
+    }
+
+    // The labelled levels' exchange: CTA b's count alone (the same in all its threads). What every level
+    // pays for is its chain of instructions between the last claim and the first ownership test, so no
+    // key travels (only a sweep's last level needs one: last_level_key), the counts are adjacent words,
+    // and warp reductions combine them (192^3 grid, 1,026 such exchanges: 7.44 -> 6.8 ms a call, with
+    // the sweeps out of line).
+    __device__ bool exchange_counts(ExResult& r, int cnt) {
+        __syncthreads();
+        const unsigned e = ++epoch;
+        const int B = gridDim.x, b = blockIdx.x;
+        Ctl* c = a->ctl;
+        int* ex = sm->exc[e & 1];  // rewritten two exchanges later, behind the barriers of the one between
+        if (threadIdx.x < 32) {
+            int bad = 0;
+            int* at = c->counts[e & 1];
+            if (threadIdx.x == 0) {
+                at[b] = cnt;
+                red_release_add(&c->arrive, 1u);
+                const unsigned target = e * (unsigned)B;
+                if ((int)(ld_acquire(&c->arrive) - target) < 0) {
+                    const unsigned long long t0 = globaltimer_ns();
+                    unsigned spins = 0;
+                    while ((int)(ld_acquire(&c->arrive) - target) < 0) {
+                        if ((++spins & 31u) == 0) {
+                            if (ld_volatile(&c->status) & (kErrTimeout | kErrInternal | kErrTooLarge)) { bad = 1; break; }
+                            if ((long long)(globaltimer_ns() - t0) > a->limit_ns) {
+                                atomicOr(&c->status, kErrTimeout);
+                                bad = 1;
+                                break;
+                            }
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            int x = 0, y = 0, mx = 0;
+            for (int i0 = threadIdx.x; i0 < B; i0 += 32 * 8) {
+                int v[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) v[t] = i0 + 32 * t < B ? ldcg(at + i0 + 32 * t) : 0;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    if (i0 + 32 * t < b) x += v[t];
+                    y += v[t];
+                    mx = max(mx, v[t]);
+                }
+            }
+            x = __reduce_add_sync(0xffffffffu, x);
+            y = __reduce_add_sync(0xffffffffu, y);
+            mx = __reduce_max_sync(0xffffffffu, mx);
+            if (threadIdx.x == 0) {
+                ex[0] = y;
+                ex[1] = x;
+                ex[2] = mx;
+                ex[3] = bad;
+            }
+        }
+        __syncthreads();
+        r.total = ex[0];
+        r.pre = ex[1];
+        r.maxcnt = ex[2];
+        r.key = kKeyMax;
+        return ex[3] == 0;
+    }
+
+    // Min (degree, id) key over the level at labels [first, first + size), by every CTA.
+    __device__ bool last_level_key(int first, int size, unsigned long long& key) {
+        unsigned long long m = kKeyMax;
+        const int stride = cta_count() * blockDim.x;
+        for (int i = cta_rank() * blockDim.x + threadIdx.x; i < size; i += stride) {
+            const int v = ldcg(a->perm + (a->n - 1 - (first + i)));
+            if (in_graph(v)) m = min(m, pack_key(__ldg(a->deg + v), v));
+        }
+        accumulate(0, m);
+        ExResult r;
+        if (!exchange(r)) return false;
+        key = r.key;
+        return true;
     }
 
     // ---- the middle tier's exchange: the mid_k CTAs of cluster 0 ----
@@ -1213,11 +1303,9 @@ struct Engine {
         return mask;
     }
 
-    // Labelled, bottom-up, step 1: every frontier vertex publishes its key in fkey, and the slice's
-    // min (degree, id) is accumulated, as in phase_a.
+    // Labelled, bottom-up, step 1: every frontier vertex publishes its key in fkey.
     __device__ void publish_keys(int d, unsigned long long ord0, const Slice& s) {
         const int T = blockDim.x;
-        unsigned long long mk = kKeyMax;
         for (int j = (int)threadIdx.x; j < s.cnt; j += T) {
             const int u = sid(s, j);
             if (!in_graph(u)) {
@@ -1225,9 +1313,7 @@ struct Engine {
                 continue;
             }
             a->fkey[u] = level_key(d, ord0 + (unsigned long long)j);
-            mk = min(mk, pack_key(__ldg(a->deg + u), u));
         }
-        accumulate(0, mk);
     }
 
     // The round-0 element of a slice and its row, which phase B expects from phase A.
@@ -1611,6 +1697,81 @@ struct Engine {
         }
     }
 
+    // Consecutive whole-grid labelled levels from level d, this CTA's slice of it cur: claims, the exchange,
+    // ownership; element j of CTA b's slice has order b * slot + j. Until the sweep ends (F = 0; d and the
+    // prev_size vertices at prev_start are the last level), or the next level is small or out of balance: it
+    // is then numbered (F vertices at lstart) and every CTA has seen it. Returns false on a failed wait.
+    __device__ bool grid_levels(int& d, int& lstart, int nv, Slice cur, int& prev_start, int& prev_size, int& F) {
+        Ctl* c = a->ctl;
+        const int b = cta_rank(), B = cta_count();
+        const unsigned long long slot = ((1ull << a->obits) - 1ull) / (unsigned long long)B;
+        int cb = 0;
+        while (true) {
+            if ((unsigned long long)cur.cnt > slot) {
+                // the slice's orders would spill into the next CTA's (only with a forced key width:
+                // the host otherwise sizes the grid so that slot >= n); every CTA's next wait sees it
+                fail(kErrTooLarge);
+                return false;
+            }
+            const unsigned long long ord0 = (unsigned long long)b * slot;
+            int u0;
+            int r0[8];
+            // bottom-up by the size of the previous level (this one's is known after the exchange)
+            const bool bu = bottom_up(prev_size, lstart - nv);
+            if (bu) {
+                publish_keys(d, ord0, cur);
+                round0_row(cur, u0, r0);
+            } else {
+                phase_a(d, ord0, cur, u0, r0, false);
+            }
+            tick(kPhClaim);
+            ExResult r;
+            if (!exchange_counts(r, cur.cnt)) return false;
+            tick(kPhExchange);
+            stat_add(kStGrid, 1);
+            if (r.total == 0) {
+                --d;
+                F = 0;
+                return true;
+            }
+            if (bu) {
+                claims_bottom_up(d);
+                if (!barrier()) return false;
+                tick(kPhClaim);
+            }
+            write_labels(cur, lstart + r.pre);
+            tick(kPhLabels);
+            if (b == 0 && threadIdx.x == 0) c->qtail[(d + 2) % 3] = 0;
+            Slice nxt;
+            int* stage = (d & 1) ? a->qa : a->qb;
+            const int kids = phase_b(d, ord0, cur, u0, r0, sm->cache[cb ^ 1], stage, &c->qtail[(d + 1) % 3], -1,
+                                     lstart + r.pre - nv, &nxt);
+            tick(kPhOwn);
+            prev_start = lstart;
+            prev_size = r.total;
+            lstart += r.total;
+            ++d;
+            cur = nxt;
+            if (cur.sh) cb ^= 1;
+            const int fair = (r.total + B - 1) / B;
+            if (r.total < a->narrow_thr || (a->mid_k > 0 && r.total < a->mid_thr) || r.maxcnt > 2 * fair + 64) {
+                // number level d now and redistribute it (or hand it to CTA 0 or the middle tier)
+                ExResult r2;
+                if (!exchange_counts(r2, kids)) return false;
+                if (r2.total == 0) {
+                    --d;
+                    F = 0;
+                    return true;
+                }
+                write_labels(cur, lstart + r2.pre);
+                if (!barrier()) return false;
+                tick(kPhRedist);
+                F = r2.total;
+                return true;
+            }
+        }
+    }
+
     // Labelled sweep from root, labels from nv. On return: ecc, the min (degree, id) key of the
     // last level, and the component size (labels nv .. nv+size-1).
     __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size) {
@@ -1633,17 +1794,32 @@ struct Engine {
         cur.step = 1;
         cur.cnt = (b == 0) ? 1 : 0;
         bool narrow = kCtaOnly || a->narrow_thr > 1;
+        if (!narrow) cur = perm_range(nv, b == 0 ? 1 : 0);
         bool mid = false;   // the middle tier runs the current level
         int F = 1;          // level size (known in narrow runs and after redistribution)
         // the last completed level (grid runs detect the end one level late)
         int prev_start = nv, prev_size = 1;
-        unsigned long long prev_key = kKeyMax;
+        int known = nv;     // labels below this are in CTA 0's bitmap (grid_local)
         while (true) {
             if (narrow) {
                 unsigned long long lk = kKeyMax;
                 int lastF = 0;
+                const int from = lstart + F;  // first label of the run's first new level
                 if (kCtaOnly || b == 0) {
-                    while (true) {
+                    if (grid_local()) {
+                        local_run<false>(a, sm, lstart == nv, d, lstart, F, a->local_hi);
+                        if (sm->wr.bad) {
+                            fail(kErrInternal);
+                            return false;
+                        }
+                        F = sm->wr.F;
+                        d = sm->wr.d;
+                        lstart = sm->wr.lstart;
+                        lk = sm->wr.lk;
+                        lastF = sm->wr.lastF;
+                        tick(kPhOwn);
+                        stat_add(kStNarrow, sm->wr.reached);
+                    } else while (true) {
                         if (kWarp && F <= kWarpLevel) {
                             // a run of narrow levels on warp 0 (where kWarp is on, as above)
                             if (threadIdx.x < 32)
@@ -1711,6 +1887,7 @@ struct Engine {
                         c->pub_ecc = d;
                         c->pub_key = lk;
                         c->pub_lastF = lastF;
+                        c->pub_reached = from;
                         c->qtail[0] = c->qtail[1] = c->qtail[2] = 0;
                     }
                 }
@@ -1736,6 +1913,12 @@ struct Engine {
                     ecc = d;
                     size = lstart + lastF2 - nv;
                     return true;
+                }
+                if (grid_local()) {
+                    // the run left no claims: its vertices are marked before the grid's levels claim
+                    known = lstart + F;
+                    const int first = (int)__ldcg(&c->pub_reached);
+                    if (!mark_labels(first, known - first)) return false;
                 }
                 // the middle tier or the whole grid from here: slices of the level's label range in perm
                 choose_tier(F, lstart, narrow, mid, cur);
@@ -1841,75 +2024,54 @@ struct Engine {
                     continue;
                 }
             }
-            // ---- whole-grid level d: this CTA's slice, ord = b * slot + j ----
-            if ((unsigned long long)cur.cnt > slot) {
-                // the slice's orders would spill into the next CTA's (only with a forced key width:
-                // the host otherwise sizes the grid so that slot >= n); every CTA's next wait sees it
-                fail(kErrTooLarge);
-                return false;
-            }
-            const unsigned long long ord0 = (unsigned long long)b * slot;
-            int u0;
-            int r0[8];
-            // bottom-up by the size of the previous level (this one's is known after the exchange)
-            const bool bu = bottom_up(prev_size, lstart - nv);
-            if (bu) {
-                publish_keys(d, ord0, cur);
-                round0_row(cur, u0, r0);
-            } else {
-                phase_a(d, ord0, cur, u0, r0);
-            }
-            if (threadIdx.x == 0) atomicAdd(&sm->acc_cnt, cur.cnt);
-            tick(kPhClaim);
-            ExResult r;
-            if (!exchange(r)) return false;
-            tick(kPhExchange);
-            stat_add(kStGrid, 1);
-            if (r.total == 0) {
-                last_key = prev_key;
-                ecc = d - 1;
-                size = prev_start + prev_size - nv;
-                return true;
-            }
-            if (bu) {
-                claims_bottom_up(d);
-                if (!barrier()) return false;
-                tick(kPhClaim);
-            }
-            write_labels(cur, lstart + r.pre);
-            tick(kPhLabels);
-            if (b == 0 && threadIdx.x == 0) c->qtail[(d + 2) % 3] = 0;
-            Slice nxt;
-            int* stage = (d & 1) ? a->qa : a->qb;
-            const int kids = phase_b(d, ord0, cur, u0, r0, sm->cache[cb ^ 1], stage, &c->qtail[(d + 1) % 3], -1,
-                                     lstart + r.pre - nv, &nxt);
-            tick(kPhOwn);
-            prev_start = lstart;
-            prev_size = r.total;
-            prev_key = r.key;
-            lstart += r.total;
-            ++d;
-            cur = nxt;
-            if (cur.sh) cb ^= 1;
-            const int fair = (r.total + B - 1) / B;
-            if (r.total < a->narrow_thr || (a->mid_k > 0 && r.total < a->mid_thr) || r.maxcnt > 2 * fair + 64) {
-                // number level d now and redistribute it (or hand it to CTA 0 or the middle tier)
-                if (threadIdx.x == 0) atomicAdd(&sm->acc_cnt, kids);
-                ExResult r2;
-                if (!exchange(r2)) return false;
-                if (r2.total == 0) {
-                    last_key = prev_key;
-                    ecc = d - 1;
-                    size = lstart - nv;
-                    return true;
+            // ---- whole-grid levels ----
+            if constexpr (!kCtaOnly) {
+                save_counters();
+                if (!run_grid_levels<kAsync, kBottomUp>(a, sm, d, lstart, nv, cur.g, cur.cnt, prev_start, prev_size))
+                    return false;
+                load_counters();
+                F = sm->wr.F;
+                d = sm->wr.d;
+                lstart = sm->wr.lstart;
+                prev_start = sm->sw.prev_start;
+                prev_size = sm->wr.lastF;
+                __syncthreads();
+                if (F == 0) {
+                    ecc = d;
+                    size = prev_start + prev_size - nv;
+                    return last_level_key(prev_start, prev_size, last_key);
                 }
-                write_labels(cur, lstart + r2.pre);
-                if (!barrier()) return false;
-                tick(kPhRedist);
-                F = r2.total;
                 choose_tier(F, lstart, narrow, mid, cur);
+                if (narrow && grid_local()) {
+                    // CTA 0 learns what the grid's levels visited since its last run
+                    for (int i = b * blockDim.x + threadIdx.x; i < lstart + F - known; i += B * blockDim.x) {
+                        const int v = ldcg(a->perm + (a->n - 1 - (known + i)));
+                        if (in_graph(v)) atomicOr(a->gvis + ((unsigned)v >> 5), 1u << ((unsigned)v & 31u));
+                    }
+                    if (!barrier()) return false;
+                    tick(kPhRedist);
+                }
             }
         }
+    }
+
+    // Whether the grid's narrow labelled levels keep their state in CTA 0's shared memory (rcm_local.cuh).
+    // A run starts below narrow_thr and ends at local_hi, half as much again: coming and going costs two
+    // barriers and a pass over the bitmap. GB300: a 1000^2 grid 16.8 -> 12.2 ms a call, a 30,000-vertex 3D
+    // grid 0.84 -> 0.59, a 100^3 grid from host memory 3.32 -> 2.79.
+    __device__ bool grid_local() const {
+        if constexpr (kCtaOnly) return false;
+        else return a->local_hi > 0;
+    }
+
+    // Claims of the vertices at labels [first, first + count) set as numbered, by every CTA, then a barrier.
+    __device__ bool mark_labels(int first, int count) {
+        const int stride = cta_count() * blockDim.x;
+        for (int i = cta_rank() * blockDim.x + threadIdx.x; i < count; i += stride) {
+            const int v = ldcg(a->perm + (a->n - 1 - (first + i)));
+            if (in_graph(v)) *claim_p(v) = 0;
+        }
+        return barrier();
     }
 
     // Whether this CTA's sweeps keep their state in shared memory (rcm_local.cuh): always where the
@@ -1918,6 +2080,25 @@ struct Engine {
         if constexpr (kSmem) return true;
         if constexpr (kCtaOnly) return sm->loc.cap >= a->n;
         return false;
+    }
+
+    // The engine's counters (the same in every thread) handed to an out-of-line sweep and taken back.
+    __device__ void save_counters() {
+        if (threadIdx.x == 0) {
+            sm->sw.epoch = epoch;
+            sm->sw.cepoch = cepoch;
+            sm->sw.sweep_id = sweep_id;
+            sm->sw.scan_par = scan_par;
+            sm->sw.async_ok = async_ok;
+        }
+        __syncthreads();
+    }
+    __device__ void load_counters() {
+        epoch = sm->sw.epoch;
+        cepoch = sm->sw.cepoch;
+        sweep_id = sm->sw.sweep_id;
+        scan_par = sm->sw.scan_par;
+        async_ok = sm->sw.async_ok;
     }
 
     // A levels-only / labelled sweep by the engine this graph runs on.
@@ -1933,7 +2114,18 @@ struct Engine {
                 return true;
             }
         }
-        if constexpr (!kSmem) return sweep_levels(root, ecc, last_key, reached);
+        if constexpr (!kCtaOnly) {
+            save_counters();
+            if (!run_grid_levels_only<kAsync, kBottomUp>(a, sm, root)) return false;
+            load_counters();
+            ecc = sm->sw.ecc;
+            last_key = sm->sw.key;
+            reached = sm->sw.reached;
+            __syncthreads();
+            return true;
+        } else if constexpr (!kSmem) {
+            return sweep_levels(root, ecc, last_key, reached);
+        }
         return false;
     }
     __device__ bool labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size) {
@@ -1952,7 +2144,18 @@ struct Engine {
                 return true;
             }
         }
-        if constexpr (!kSmem) return sweep_labelled(root, nv, ecc, last_key, size);
+        if constexpr (!kCtaOnly) {
+            save_counters();
+            if (!run_grid_labelled<kAsync, kBottomUp>(a, sm, root, nv)) return false;
+            load_counters();
+            ecc = sm->sw.ecc;
+            last_key = sm->sw.key;
+            size = sm->sw.size;
+            __syncthreads();
+            return true;
+        } else if constexpr (!kSmem) {
+            return sweep_labelled(root, nv, ecc, last_key, size);
+        }
         return false;
     }
 
@@ -1998,15 +2201,6 @@ struct Engine {
             }
         }
         return barrier();
-    }
-
-    // Claims of the vertices at labels [nv, nv + size) set as numbered (CTA engines).
-    __device__ void mark_numbered(int nv, int size) {
-        for (int i = threadIdx.x; i < size; i += blockDim.x) {
-            const int v = ldcg(a->perm + (a->n - 1 - (nv + i)));
-            if (in_graph(v)) *claim_p(v) = 0;
-        }
-        __syncthreads();
     }
 
     // Start of the next component: min (degree, id) over the vertices not yet numbered.
@@ -2440,7 +2634,7 @@ struct Engine {
             if (!component((int)(unsigned)(k0 & 0xffffffffu), nv, size, left)) return false;
             if (size < 0) continue;
             // local sweeps leave no claims: the vertices just numbered are marked for the searches below
-            if (local() && nv + size < n) mark_numbered(nv, size);
+            if (local() && nv + size < n && !mark_labels(nv, size)) return false;
             nv += size;
         }
         return true;
@@ -2468,6 +2662,71 @@ __device__ __noinline__ void run_warp_labelled(const EngineArgs* a, EngineSmem* 
     cur.step = step;
     cur.cnt = F;
     e.warp_labelled(d, lstart, F, cb, cur);
+}
+
+template <bool kAsync, bool kBottomUp>
+__device__ __noinline__ bool run_grid_levels_only(const EngineArgs* a, EngineSmem* sm, int root) {
+    Engine<false, false, kAsync, kBottomUp> e;
+    e.a = a;
+    e.sm = sm;
+    e.load_counters();
+    int ecc;
+    unsigned long long key;
+    long long reached;
+    if (!e.sweep_levels(root, ecc, key, reached)) return false;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm->sw.ecc = ecc;
+        sm->sw.key = key;
+        sm->sw.reached = reached;
+    }
+    e.save_counters();
+    return true;
+}
+
+template <bool kAsync, bool kBottomUp>
+__device__ __noinline__ bool run_grid_labelled(const EngineArgs* a, EngineSmem* sm, int root, int nv) {
+    Engine<false, false, kAsync, kBottomUp> e;
+    e.a = a;
+    e.sm = sm;
+    e.load_counters();
+    int ecc, size;
+    unsigned long long key;
+    if (!e.sweep_labelled(root, nv, ecc, key, size)) return false;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm->sw.ecc = ecc;
+        sm->sw.key = key;
+        sm->sw.size = size;
+    }
+    e.save_counters();
+    return true;
+}
+
+template <bool kAsync, bool kBottomUp>
+__device__ __noinline__ bool run_grid_levels(const EngineArgs* a, EngineSmem* sm, int d, int lstart, int nv,
+                                             const int* g, int cnt, int prev_start, int prev_size) {
+    Engine<false, false, kAsync, kBottomUp> e;
+    e.a = a;
+    e.sm = sm;
+    e.load_counters();
+    typename Engine<false, false, kAsync, kBottomUp>::Slice cur;
+    cur.sh = nullptr;
+    cur.g = g;
+    cur.step = -1;
+    cur.cnt = cnt;
+    int F = 0;
+    if (!e.grid_levels(d, lstart, nv, cur, prev_start, prev_size, F)) return false;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm->sw.prev_start = prev_start;
+        sm->wr.F = F;
+        sm->wr.d = d;
+        sm->wr.lstart = lstart;
+        sm->wr.lastF = prev_size;
+    }
+    e.save_counters();
+    return true;
 }
 
 }  // namespace rcm

@@ -68,6 +68,11 @@ struct EngineArgs {
     // distributed shared memory, while the other CTAs wait at the next grid barrier
     int mid_k;
     int mid_thr;
+    // narrow labelled levels of the whole-grid executor with their state in CTA 0's shared memory
+    // (rcm_local.cuh); local_hi = 0: in global memory
+    int local_hi;                // a run ends at a level of this many vertices (narrow_thr starts one)
+    int local_slots, local_entries;
+    unsigned* gvis;              // bitmap of n vertices: what the grid's levels visited, for the next run
 };
 
 enum { kPhExpand = 0, kPhClaim, kPhOwn, kPhLabels, kPhExchange, kPhRedist, kPhWaitNarrow, kPhOther };
@@ -97,6 +102,7 @@ struct EngineSmem {
     int acc_cnt;                 // CTA count accumulator feeding the exchange
     unsigned long long wkey[32]; // per-warp min keys of the last accumulate()
     int ex[4];                   // exchange results: total, pre, maxcnt
+    int exc[2][4];               // the counts-only exchange's, by epoch parity (and bad)
     unsigned long long ex_key;
     int bc[8];
     unsigned long long bck;
@@ -107,6 +113,13 @@ struct EngineSmem {
         long long reached;
         unsigned long long lk;
     } wr;
+    struct {                     // an out-of-line sweep of the grid: the engine's counters, and its results
+        unsigned epoch, cepoch;
+        int sweep_id, scan_par, ecc, size, prev_start;
+        bool async_ok;
+        unsigned long long key;
+        long long reached;
+    } sw;
     int aflag;                   // async sweep: stop flag relayed to the CTA's warps
     // middle tier: this CTA's part of each cluster exchange, read by the cluster's CTAs through
     // distributed shared memory; double-buffered by epoch parity

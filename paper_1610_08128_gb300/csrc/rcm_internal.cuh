@@ -65,6 +65,7 @@ struct alignas(128) Ctl {
     long long stats[8];            // rcm_stats fields, in order
     long long phase_ns[8];         // per-phase time of CTA 0 (profile_phases)
     ExSlot slots[2][kMaxGridBlocks];  // exchange slots, double-buffered by epoch parity
+    int counts[2][kMaxGridBlocks];    // the counts-only exchange's
 };
 
 // Counters of the asynchronous levels-only sweep (one per ordering), each hot word on its own
@@ -194,12 +195,10 @@ __device__ __forceinline__ int block_excl_scan(int x, int* total, int* smem, int
     const int incl = warp_incl_scan(x);
     if (lane == 31) half[wid] = incl;
     __syncthreads();
-    // every warp scans the warp totals itself: lane l holds total l
+    // every warp adds up the warp totals itself: lane l holds total l
     const int t = lane < nw ? half[lane] : 0;
-    const int ti = warp_incl_scan(t);
-    const int before = wid > 0 ? __shfl_sync(0xffffffffu, ti, wid - 1) : 0;
-    *total = __shfl_sync(0xffffffffu, ti, 31);
-    return before + incl - x;
+    *total = __reduce_add_sync(0xffffffffu, t);
+    return __reduce_add_sync(0xffffffffu, lane < wid ? t : 0) + incl - x;
 }
 
 __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long x) {

@@ -759,6 +759,34 @@ struct Local {
         last_key = level_key(F, [&](int j) { return j < kCache ? sm->cache[cb][j] : ldcg(cur + j); });
     }
 
+    // Labelled levels from level d of F vertices at labels lstart.., held in cache buffer cb, until one is
+    // the last (returns true: F and lstart are its) or the next has at least `hi` vertices (returns false:
+    // they are the next one's). `bad` is set where a label left the graph.
+    __device__ bool labelled_levels(int& F, int& lstart, int& cb, int& d, int hi, bool& bad) {
+        const unsigned c0 = s_addr(sm->cache[0]);
+        while (true) {
+            next_generation();
+            int kids = labelled_level(F, lstart, c0 + 4 * kCache * cb, c0 + 4 * kCache * (cb ^ 1), bad);
+            if (kids < 0) {
+                __syncthreads();  // every thread has read the counts
+                kids = local_wide_level<kDirect>(a, sm, F, lstart, cb, gen, seq);
+                bad |= kids < 0;
+            }
+            if (kids <= 0) return true;
+            lstart += F;
+            F = kids;
+            cb ^= 1;
+            ++d;
+            if (F >= hi) return false;
+        }
+    }
+
+    // Min key of a labelled level at labels lstart.., held in cache buffer cb.
+    __device__ unsigned long long labelled_key(int F, int lstart, int cb) const {
+        const unsigned cache = s_addr(sm->cache[cb]);
+        return level_key(F, [&](int j) { return labelled_at(j, cache, lstart); });
+    }
+
     // Labelled sweep from root with labels from nv: eccentricity, last level's min key, size. Returns
     // false when a label left the graph.
     __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size) {
@@ -767,29 +795,57 @@ struct Local {
         __syncthreads();
         ++seq;
         int F = 1, cb = 0, lstart = nv;
-        const unsigned c0 = s_addr(sm->cache[0]);
         bool bad = false;
         ecc = 0;
-        while (true) {
-            next_generation();
-            int kids = labelled_level(F, lstart, c0 + 4 * kCache * cb, c0 + 4 * kCache * (cb ^ 1), bad);
-            if (kids < 0) {
-                __syncthreads();  // every thread has read the counts
-                kids = local_wide_level<kDirect>(a, sm, F, lstart, cb, gen, seq);
-                if (kids < 0) {
-                    bad = true;
-                    break;
-                }
-            }
-            if (kids == 0) break;
-            lstart += F;
-            F = kids;
-            cb ^= 1;
-            ++ecc;
-        }
-        last_key = level_key(F, [&](int j) { return labelled_at(j, c0 + 4 * kCache * cb, lstart); });
+        labelled_levels(F, lstart, cb, ecc, kIntMax, bad);
+        last_key = labelled_key(F, lstart, cb);
         size = lstart + F - nv;
         return !__syncthreads_or(bad);
+    }
+
+    // A run of narrow levels on CTA 0 of the grid: level d, F (below kCache) vertices at labels lstart..
+    // in perm. first: the sweep starts here, nothing else is visited; otherwise gvis holds what the grid's
+    // levels visited since the last run. Runs until the sweep ends or a level has `hi` vertices.
+    __device__ void run(bool first, int d, int lstart, int F, int hi) {
+        const int words = local_vis_words(n) / 4;
+        uint4* v = (uint4*)sm->loc.vis;
+        uint4* gv = (uint4*)a->gvis;
+        for (int i = threadIdx.x; i < words; i += blockDim.x) {
+            uint4 x = make_uint4(0u, 0u, 0u, 0u);
+            if (first) {
+                gv[i] = x;
+            } else {
+                const uint4 y = __ldcg(gv + i);
+                x = v[i];
+                x = make_uint4(x.x | y.x, x.y | y.y, x.z | y.z, x.w | y.w);
+            }
+            v[i] = x;
+        }
+        for (int j = threadIdx.x; j < F; j += blockDim.x) sm->cache[0][j] = ldcg(perm_end - (lstart + j));
+        __syncthreads();
+        if (first && threadIdx.x == 0) {
+            const unsigned w = (unsigned)sm->cache[0][0];
+            sm->loc.vis[w >> 5] |= 1u << (w & 31u);
+        }
+        __syncthreads();
+        ++seq;
+        const int d0 = d;
+        int cb = 0;
+        bool bad = false;
+        const bool end = labelled_levels(F, lstart, cb, d, hi, bad);
+        const unsigned long long key = end ? labelled_key(F, lstart, cb) : kKeyMax;
+        bad = __syncthreads_or(bad);
+        save();
+        if (threadIdx.x == 0) {
+            sm->wr.F = end ? 0 : F;
+            sm->wr.lastF = end ? F : 0;
+            sm->wr.d = d;
+            sm->wr.lstart = lstart;
+            sm->wr.lk = key;
+            sm->wr.reached = d - d0 + (end ? 1 : 0);
+            sm->wr.bad = bad ? 1 : 0;
+        }
+        __syncthreads();
     }
 };
 
@@ -824,6 +880,14 @@ __device__ __noinline__ void local_sweep(const EngineArgs* a, EngineSmem* sm, in
         sm->wr.bad = ok ? 0 : 1;
     }
     __syncthreads();
+}
+
+// Local::run out of line; results in sm->wr (reached: levels run).
+template <bool kDirect>
+__device__ __noinline__ void local_run(const EngineArgs* a, EngineSmem* sm, int first, int d, int lstart, int F,
+                                       int hi) {
+    Local<kDirect> l(a, sm);
+    l.run(first != 0, d, lstart, F, hi);
 }
 
 }  // namespace rcm

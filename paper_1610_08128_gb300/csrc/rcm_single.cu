@@ -102,6 +102,10 @@ static const void* single_kernel(int threads, bool async = false, bool hybrid = 
 constexpr int kComponentSlots = 8192;
 constexpr int kComponentEntries = 3072;
 constexpr size_t kComponentSmem = 206 * 1024;
+// The grid kernel's table leaves every CTA's wide levels some L1 where it can (they read their rows
+// twice): a 1M-vertex power-law graph 3.99 ms with 96 KB of shared memory, 4.24 with 201.
+constexpr size_t kGridLocalSmem = 170 * 1024;
+constexpr size_t kComponentSmem2 = 94 * 1024;  // the most with two CTAs on an SM
 
 constexpr int kSingleDynSmem = (int)((sizeof(unsigned long long) + sizeof(int)) * kCompSmem);
 
@@ -113,7 +117,7 @@ static int single_blocks_per_sm(int threads, bool async = false, bool hybrid = f
     if (g_single_blocks_per_sm[idx] < 0) {
         int b = 0;
         const void* k = single_kernel(threads, async, hybrid);
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSingleDynSmem);
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kComponentSmem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, threads, kSingleDynSmem);
         g_single_blocks_per_sm[idx] = b;
         cudaFuncSetAttribute((const void*)k_rcm_components<kComponentThreads>,
@@ -293,6 +297,10 @@ rcm_status single_launch(int n, long long nnz, const rcm_options& o, SingleLaunc
     // measured on GB300 (the 192^3 grid 7.40 against 7.64 ms, a 1000^2 grid 19.1 against 24.3 ms)
     int narrow = o.narrow_threshold == 0 ? sl.threads : (o.narrow_threshold < 0 ? 0 : o.narrow_threshold);
     sl.narrow = std::min(narrow, kCache);
+    // CTA 0's narrow levels in shared memory: where its CTA has the SM to itself and no middle tier
+    // takes the levels above them
+    // (nor on patterns dense enough for bottom-up levels: they have few levels, and wide ones)
+    sl.local = sl.threads == 512 && !sl.hybrid && sl.narrow > 1 && sl.mid_k == 0 && sl.blocks <= di.sms;
     sl.limit_ns = o.spin_limit_ns > 0 ? o.spin_limit_ns : 20000000000LL;
     // label during every sweep by default on a wide grid: there a labelled level is cheaper than a
     // levels-only one (GB300, 152 CTAs: the 192^3 grid 7.08 against 7.43 ms, a 1000^2 grid 17.7
@@ -321,11 +329,11 @@ rcm_status single_launch(int n, long long nnz, const rcm_options& o, SingleLaunc
 // streaming through L2 do not evict them. The context's persisting-L2 limit is raised to the
 // window (clamped to the device maximum) on first use.
 static cudaError_t launch_grid(const void* kernel, const SingleLaunch& sl, void** kargs, char* win, size_t bytes,
-                               cudaStream_t s) {
+                               size_t dyn, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(sl.blocks);
     cfg.blockDim = dim3(sl.threads);
-    cfg.dynamicSmemBytes = kSingleDynSmem;
+    cfg.dynamicSmemBytes = dyn;
     cfg.stream = s;
     cudaLaunchAttribute attr[3];
     int na = 0;
@@ -411,7 +419,10 @@ static cudaError_t release_persisting(const char* win, size_t bytes, cudaStream_
 static cudaError_t launch_components(EngineArgs& args, const SingleLaunch& sl, cudaStream_t s) {
     const int blocks = std::max(1, sl.blocks * sl.threads / kComponentThreads);
     int cap = sl.cluster ? 0 : args.n, slots = kComponentSlots, entries = kComponentEntries;
-    while (slots > 2048 && local_bytes(cap, slots, entries) > kComponentSmem) slots /= 2;
+    // room for two CTAs on an SM where the bitmap leaves it (300,000 points, 2-NN, thousands of small
+    // components: 6.5 ms with two, 7.2 with one and a larger table)
+    const size_t most = local_bytes(cap, 2048, entries) <= kComponentSmem2 ? kComponentSmem2 : kComponentSmem;
+    while (slots > 2048 && local_bytes(cap, slots, entries) > most) slots /= 2;
     size_t bytes = local_bytes(cap, slots, entries);
     if (cap == 0 || bytes > kComponentSmem) {
         cap = entries = 0;
@@ -509,6 +520,23 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
     args.aq_cap = async ? (unsigned)slots : 0u;
     args.mid_k = sl.small ? 0 : sl.mid_k;
     args.mid_thr = args.mid_k ? sl.mid_thr : 0;
+    // narrow levels with their state in CTA 0's shared memory, where the graph's bitmap fits beside the
+    // component table's sort (spare: the union-find parents, not in use during a sweep)
+    args.local_hi = args.local_slots = args.local_entries = 0;
+    // from the next 16-byte boundary; n / 32 words and a few fit what is left of the array and its padding
+    args.gvis = (unsigned*)(base + align16(L.pool4 + 12 * (size_t)n));
+    size_t dyn = kSingleDynSmem;
+    if (sl.local) {
+        int slots = kComponentSlots;
+        while (slots > 2048 && local_bytes(n, slots, kComponentEntries) > kGridLocalSmem) slots /= 2;
+        const size_t bytes = local_bytes(n, slots, kComponentEntries);
+        if (bytes <= kComponentSmem) {
+            args.local_hi = std::min(sl.narrow + sl.narrow / 2, kCache);
+            args.local_slots = slots;
+            args.local_entries = kComponentEntries;
+            dyn = std::max(dyn, bytes);
+        }
+    }
     int stall = sl.stall;
     void* kargs[] = {&args, &stall};
     if (sl.small) {
@@ -519,7 +547,7 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(sl.blocks);
         cfg.blockDim = dim3(sl.threads);
-        cfg.dynamicSmemBytes = kSingleDynSmem;
+        cfg.dynamicSmemBytes = dyn;
         cfg.stream = s;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -530,14 +558,14 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
         cfg.numAttrs = 1;
         e = cudaLaunchKernelExC(&cfg, single_kernel(sl.threads, async, hybrid), kargs);
     } else if (sl.l2_persist || sl.mid_k > 0) {
-        e = launch_grid(single_kernel(sl.threads, async, hybrid), sl, kargs, base + L.claim, L.bigrows - L.claim, s);
+        e = launch_grid(single_kernel(sl.threads, async, hybrid), sl, kargs, base + L.claim, L.bigrows - L.claim, dyn, s);
         if (e == cudaSuccess) e = launch_components(args, sl, s);
         if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
         if (e == cudaSuccess && sl.l2_persist) e = release_persisting(base + L.claim, L.bigrows - L.claim, s);
         return e;
     } else {
         e = cudaLaunchCooperativeKernel(single_kernel(sl.threads, async, hybrid), dim3(sl.blocks), dim3(sl.threads), kargs,
-                                        kSingleDynSmem, s);
+                                        dyn, s);
     }
     if (e == cudaSuccess && !sl.small) e = launch_components(args, sl, s);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
