@@ -353,23 +353,15 @@ rcm_status rcm_bandwidth_profile(int32_t n, const int32_t* rowptr, const int32_t
     if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, 256, s);
     if (e == cudaSuccess) {
         k_bw_scatter<<<grid, pb, 0, s>>>(n, perm, pos, err);
+        k_bw_rows<<<grid, pb, 0, s>>>(n, rowptr, colidx, pos, err, out);
         e = cudaGetLastError();
     }
     unsigned long long h[3] = {0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, out, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && (h[2] & 0xffffffffu) != 0) {
-        ws_free(buf, s);
-        return RCM_ERR_INVALID_ARG;
-    }
-    if (e == cudaSuccess) {
-        k_bw_rows<<<grid, pb, 0, s>>>(n, rowptr, colidx, perm, pos, out);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, out, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
     ws_free(buf, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_status(e);
+    if ((h[2] & 0xffffffffu) != 0) return RCM_ERR_INVALID_ARG;  // not a permutation
     *bw = (int64_t)h[0];
     *profile = (int64_t)h[1];
     return RCM_OK;

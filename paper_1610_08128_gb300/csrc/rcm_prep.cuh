@@ -181,7 +181,7 @@ __global__ void k_sort_rows_big(int n, const int* __restrict__ rowptr, const int
 __global__ void k_bw_scatter(int n, const int* __restrict__ perm, int* __restrict__ pos, int* __restrict__ err);
 
 __global__ void k_bw_rows(int n, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                          const int* __restrict__ perm, const int* __restrict__ pos,
+                          const int* __restrict__ pos, int* __restrict__ err,
                           unsigned long long* __restrict__ out);
 
 }  // namespace rcm
