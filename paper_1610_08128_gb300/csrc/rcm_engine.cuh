@@ -82,6 +82,17 @@ template <bool kCtaOnly, bool kSmem, bool kAsync, bool kBottomUp, bool kWarp>
 __device__ __noinline__ void run_warp_labelled(const EngineArgs* a, EngineSmem* sm, int d, int lstart, int F, int cb,
                                                const int* sh, const int* g, int step);
 
+// Phases A and B for the entries beyond the padded rows of a warp's vertices (u < 0: none on this lane),
+// out of line: most graphs have none, and inlined they cost every level registers (192^3 grid 7.05 against
+// 6.6 ms). Claims; the number of children owned there; those written from position pos on.
+template <class Eng>
+__device__ __noinline__ void long_claims(const EngineArgs* a, int u, int dg, unsigned long long key);
+template <class Eng>
+__device__ __noinline__ int long_owned(const EngineArgs* a, int u, int dg, unsigned long long key);
+template <class Eng>
+__device__ __noinline__ void long_children(const EngineArgs* a, int u, int dg, unsigned long long key, int pos, int* dst,
+                                           int lab_base);
+
 // The whole grid's sweeps and, inside the labelled one, its runs of whole-grid levels, out of line: one
 // copy each, with registers of its own (inlined into one kernel they spill: 192^3 grid 7.1 against 6.8
 // ms). Results in sm->sw and sm->wr.
@@ -233,33 +244,49 @@ struct Engine {
         }
     }
 
-    // The same for the ownership tests of phase B: each round's entries come with their claims,
-    // fn(src, w, claim) (claim = kClaimNone past the row's end), and the entries of kLongRounds
-    // rounds, then their claims, are loaded before any is used: a hub costs two dependent round
-    // trips per kLongRounds rounds, not per round.
-    template <class Fn>
-    __device__ void for_long_rows_claims(bool has, int u, int dg, Fn fn) const {
-        unsigned pend = __ballot_sync(0xffffffffu, has && dg > kEllNb);
+    // Whether a lane of the warp holds a long row (u < 0: it holds no vertex).
+    __device__ bool any_long(int u, int dg) const { return __any_sync(0xffffffffu, u >= 0 && dg > kEllNb); }
+
+    // The same with the lanes' long rows laid end to end and read 32 entries per round, whatever row they
+    // belong to: on a scale-free graph most rows are a few entries over, and a warp's 32 such rows cost a
+    // few rounds instead of 32 (1M vertices, mean degree 10, GB300: see the hub defaults). No early stop.
+    // fn(src, w, cw, mine, head): the entry's lane and vertex (-1 past the end); with kClaims its claim
+    // (else kClaimNone); this lane's own row's entries in the round, as a mask of lanes; and the first lane
+    // of the round that holds an entry of the same row as this lane's.
+    template <bool kClaims, class Fn>
+    __device__ void for_long_flat(bool has, int u, int dg, Fn fn) const {
+        const int over = has && dg > kEllNb ? dg - kEllNb : 0;
+        if (!__any_sync(0xffffffffu, over)) return;
         const int lane = threadIdx.x & 31;
-        while (pend) {
-            const int src = __ffs(pend) - 1;
-            pend &= pend - 1;
-            const int uu = __shfl_sync(0xffffffffu, u, src);
-            const int dd = __shfl_sync(0xffffffffu, dg, src);
-            const int* row = a->adj + __ldg(a->rowptr + uu);
-            for (int k0 = kEllNb; k0 < dd; k0 += 32 * kLongRounds) {
-                int w[kLongRounds];
-                unsigned long long c[kLongRounds];
+        const int end = warp_incl_scan(over), begin = end - over;
+        const int total = __shfl_sync(0xffffffffu, end, 31);
+        // where this lane's row would start if entry 0 were the warp's first
+        const int at = (over ? __ldg(a->rowptr + u) + kEllNb : 0) - begin;
+        for (int e0 = 0; e0 < total; e0 += 32 * kLongRounds) {
+            int w[kLongRounds], src[kLongRounds];
 #pragma unroll
-                for (int r = 0; r < kLongRounds; ++r) {
-                    const int k = k0 + 32 * r + lane;
-                    w[r] = k < dd ? __ldg(row + k) : -1;
-                }
+            for (int r = 0; r < kLongRounds; ++r) {
+                const int e = e0 + 32 * r + lane;
+                // the first lane whose rows end beyond e
+                int l = 0;
 #pragma unroll
-                for (int r = 0; r < kLongRounds; ++r) c[r] = w[r] >= 0 ? ld_claim(w[r]) : kClaimNone;
+                for (int s = 16; s > 0; s >>= 1)
+                    if (__shfl_sync(0xffffffffu, end, l + s - 1) <= e) l += s;
+                src[r] = l;
+                const int p = __shfl_sync(0xffffffffu, at, l) + e;
+                w[r] = e < total ? __ldg(a->adj + p) : -1;
+            }
+            unsigned long long c[kLongRounds];
 #pragma unroll
-                for (int r = 0; r < kLongRounds; ++r)
-                    if (k0 + 32 * r < dd) fn(src, w[r], c[r]);
+            for (int r = 0; r < kLongRounds; ++r) c[r] = kClaims && w[r] >= 0 ? ld_claim(w[r]) : kClaimNone;
+#pragma unroll
+            for (int r = 0; r < kLongRounds; ++r) {
+                const int first = e0 + 32 * r;
+                if (first >= total) break;
+                const int lo = max(begin - first, 0), hi = min(end - first, 32);
+                const unsigned mine = hi > lo ? (hi >= 32 ? 0xffffffffu : (1u << hi) - 1u) & ~((1u << lo) - 1u) : 0u;
+                const int head = max(__shfl_sync(0xffffffffu, begin, src[r]) - first, 0);
+                fn(src[r], w[r], c[r], mine, head);
             }
         }
     }
@@ -590,7 +617,7 @@ struct Engine {
             }
             // neighbours beyond the padded row (degree > 7), a warp round at a time; the new ones of
             // a round take consecutive positions reserved by one atomic
-            for_long_rows(u >= 0, u, d, [&](int, int w) {
+            for_long_flat<false>(u >= 0, u, d, [&](int, int w, unsigned long long, unsigned, int) {
                 const bool fresh = w >= 0 && atomicExch(vis_p(w), s) != s;
                 const unsigned bal = __ballot_sync(0xffffffffu, fresh);
                 if (bal) {
@@ -606,7 +633,6 @@ struct Engine {
                     }
                     if (lane == 0) cnt += __popc(bal);
                 }
-                return false;
             });
             const int c = __popc(mask);
             int tot;
@@ -1398,11 +1424,7 @@ struct Engine {
                     }
                 }
             }
-            for_long_rows(u >= 0, u, dg, [&](int src, int w) {
-                const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
-                if (w >= 0) atomicMin(claim_p(w), kk);
-                return false;
-            });
+            if (any_long(u, dg)) long_claims<Engine>(a, u, dg, key);
         }
         if (with_key) accumulate(0, mk);
     }
@@ -1445,11 +1467,7 @@ struct Engine {
                     u = -1;
                 }
             }
-            for_long_rows_claims(u >= 0, u, dg, [&](int src, int w, unsigned long long cw) {
-                const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
-                const int m = __popc(__ballot_sync(0xffffffffu, w >= 0 && cw == kk));
-                if ((int)(threadIdx.x & 31) == src) c += m;
-            });
+            if (any_long(u, dg)) c += long_owned<Engine>(a, u, dg, key);
             int tot;
             const int ex = cta_scan(c, &tot);
             if (j0 == 0) {
@@ -1511,23 +1529,7 @@ struct Engine {
             }
             // the rest of a long row, in row order: a round's owned entries take consecutive
             // positions after the owner's earlier children
-            for_long_rows_claims(u >= 0, u, dg, [&](int src, int w, unsigned long long cw) {
-                const int lane = threadIdx.x & 31;
-                const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
-                const bool own = w >= 0 && cw == kk;
-                const unsigned bal = __ballot_sync(0xffffffffu, own);
-                const int base = __shfl_sync(0xffffffffu, pos, src);
-                if (own) {
-                    const int p = base + __popc(bal & ((1u << lane) - 1u));
-                    prefetch_row(w);
-                    dst[p] = w;
-                    if (lab_base >= 0) {
-                        const int lab = lab_base + p;
-                        if ((unsigned)lab < (unsigned)n) a->perm[n - 1 - lab] = w; else fail(kErrInternal);
-                    }
-                }
-                if (lane == src) pos += __popc(bal);
-            });
+            if (any_long(u, dg)) long_children<Engine>(a, u, dg, key, pos, dst, lab_base);
         }
         __syncthreads();
         return carry;
@@ -1592,10 +1594,9 @@ struct Engine {
             // phase B: the children each vertex owns, counted, then numbered in (key, row) order
             const unsigned mask = u >= 0 ? owned_mask(rw, dg, key) : 0u;
             int cnt = __popc(mask);
-            for_long_rows_claims(u >= 0, u, dg, [&](int src, int w, unsigned long long cw) {
+            for_long_flat<true>(u >= 0, u, dg, [&](int src, int w, unsigned long long cw, unsigned mine, int) {
                 const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
-                const int m = __popc(__ballot_sync(0xffffffffu, w >= 0 && cw == kk));
-                if (lane == src) cnt += m;
+                cnt += __popc(__ballot_sync(0xffffffffu, w >= 0 && cw == kk) & mine);
             });
             const int incl = warp_incl_scan(cnt);
             const int kids = __shfl_sync(0xffffffffu, incl, 31);
@@ -1614,19 +1615,19 @@ struct Engine {
                         ++q;
                     }
             }
-            for_long_rows_claims(u >= 0, u, dg, [&](int src, int w, unsigned long long cw) {
+            for_long_flat<true>(u >= 0, u, dg, [&](int src, int w, unsigned long long cw, unsigned mine, int head) {
                 const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
                 const bool own = w >= 0 && cw == kk;
                 const unsigned bal = __ballot_sync(0xffffffffu, own);
                 const int base = __shfl_sync(0xffffffffu, q, src);
                 if (own) {
-                    const int qq = base + __popc(bal & lt);
+                    const int qq = base + __popc(bal & lt & ~((1u << head) - 1u));
                     prefetch_row(w);
                     if (qq < kCache) nc[qq] = w;
                     const int lab = lab0 + qq;
                     if ((unsigned)lab < (unsigned)n) a->perm[n - 1 - lab] = w; else bad = 1;
                 }
-                if (lane == src) q += __popc(bal);
+                q += __popc(bal & mine);
             });
             __syncwarp();
             tick(kPhOwn);
@@ -2477,10 +2478,9 @@ struct Engine {
                 for (int k = 0; k < kEllNb; ++k)
                     if (k < d && r[k] < v && !cc_union(a->cc_parent, v, r[k], v0, v0 + n)) fail_at(kSiteParent, v);
             }
-            for_long_rows(open, v, d, [&](int src, int w) {
+            for_long_flat<false>(open, v, d, [&](int src, int w, unsigned long long, unsigned, int) {
                 const int vv = __shfl_sync(0xffffffffu, v, src);
                 if (w >= 0 && w < vv && !cc_union(a->cc_parent, vv, w, v0, v0 + n)) fail_at(kSiteParent, vv);
-                return false;
             });
         }
         if (!barrier()) return -2;
@@ -2662,6 +2662,53 @@ __device__ __noinline__ void run_warp_labelled(const EngineArgs* a, EngineSmem* 
     cur.step = step;
     cur.cnt = F;
     e.warp_labelled(d, lstart, F, cb, cur);
+}
+
+template <class Eng>
+__device__ __noinline__ void long_claims(const EngineArgs* a, int u, int dg, unsigned long long key) {
+    Eng e;
+    e.a = a;
+    e.template for_long_flat<false>(u >= 0, u, dg, [&](int src, int w, unsigned long long, unsigned, int) {
+        const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
+        if (w >= 0) atomicMin(e.claim_p(w), kk);
+    });
+}
+
+template <class Eng>
+__device__ __noinline__ int long_owned(const EngineArgs* a, int u, int dg, unsigned long long key) {
+    Eng e;
+    e.a = a;
+    int c = 0;
+    e.template for_long_flat<true>(u >= 0, u, dg, [&](int src, int w, unsigned long long cw, unsigned mine, int) {
+        const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
+        c += __popc(__ballot_sync(0xffffffffu, w >= 0 && cw == kk) & mine);
+    });
+    return c;
+}
+
+// In row order: a row's owned entries take consecutive positions after its owner's earlier children.
+template <class Eng>
+__device__ __noinline__ void long_children(const EngineArgs* a, int u, int dg, unsigned long long key, int pos, int* dst,
+                                           int lab_base) {
+    Eng e;
+    e.a = a;
+    const int n = a->n, lane = threadIdx.x & 31;
+    e.template for_long_flat<true>(u >= 0, u, dg, [&](int src, int w, unsigned long long cw, unsigned mine, int head) {
+        const unsigned long long kk = __shfl_sync(0xffffffffu, key, src);
+        const bool own = w >= 0 && cw == kk;
+        const unsigned bal = __ballot_sync(0xffffffffu, own);
+        const int base = __shfl_sync(0xffffffffu, pos, src);
+        if (own) {
+            const int p = base + __popc(bal & ((1u << lane) - 1u) & ~((1u << head) - 1u));
+            e.prefetch_row(w);
+            dst[p] = w;
+            if (lab_base >= 0) {
+                const int lab = lab_base + p;
+                if ((unsigned)lab < (unsigned)n) a->perm[n - 1 - lab] = w; else e.fail(kErrInternal);
+            }
+        }
+        pos += __popc(bal & mine);
+    });
 }
 
 template <bool kAsync, bool kBottomUp>
