@@ -100,7 +100,8 @@ template <bool kAsync, bool kBottomUp>
 __device__ __noinline__ bool run_grid_levels_only(const EngineArgs* a, EngineSmem* sm, int root);
 template <bool kAsync, bool kBottomUp>
 __device__ __noinline__ bool run_grid_labelled(const EngineArgs* a, EngineSmem* sm, int root, int nv);
-template <bool kAsync, bool kBottomUp>
+// kHub: with the long rows of a hub graph spread over the CTA (hub_round).
+template <bool kAsync, bool kBottomUp, bool kHub>
 __device__ __noinline__ bool run_grid_levels(const EngineArgs* a, EngineSmem* sm, int d, int lstart, int nv,
                                              const int* g, int cnt, int prev_start, int prev_size);
 
@@ -241,6 +242,57 @@ struct Engine {
                     if (!stop && k0 + 32 * r < dd) stop = fn(src, w[r]);
                 if (stop) break;
             }
+        }
+    }
+
+    // A CTA's part of a level: cnt vertex ids, element j at sh[j] (shared memory) or g[step * j]
+    // (global: a staging buffer with step 1, or a label range of perm with step -1).
+    struct Slice {
+        const int* sh;
+        const int* g;
+        int step;
+        int cnt;
+    };
+
+    __device__ int sid(const Slice& s, int j) const { return s.sh ? s.sh[j] : ldcg(s.g + (long long)s.step * j); }
+
+    // On a graph with hubs the grid spreads a round's long rows over the CTA's warps: hubs are neighbours
+    // in a level (siblings come by degree), so in label order one warp would get most of them.
+    __device__ bool hubs() const {
+        if constexpr (kCtaOnly) return false;
+        else return a->hubs != 0;
+    }
+    enum { kHubClaim, kHubCount, kHubWrite };
+    // Claims, counts or writes (from position pos on, this thread's vertex's) for the entries beyond the
+    // padded rows of the round of slice s from element j0, thread t taking element t mod 32 * warps + t / 32.
+    // Every thread calls; returns the count of this thread's own vertex.
+    template <int kWhat>
+    __device__ int hub_round(int d, unsigned long long ord0, const Slice& s, int j0, int pos, int* dst, int lab_base) {
+        const int t = (int)threadIdx.x, at = (t & 31) * (int)(blockDim.x >> 5) + (t >> 5);
+        const int j = j0 + at;
+        int u = -1, dg = 0;
+        if (j < s.cnt) {
+            u = sid(s, j);
+            if (in_graph(u)) dg = __ldg((const int*)a->ell + 8 * (size_t)u + 7);
+            else u = -1;
+        }
+        const unsigned long long key = level_key(d, ord0 + (unsigned long long)j);
+        if constexpr (kWhat == kHubClaim) {
+            if (any_long(u, dg)) long_claims<Engine>(a, u, dg, key);
+            return 0;
+        } else if constexpr (kWhat == kHubCount) {
+            sm->hub[at] = any_long(u, dg) ? long_owned<Engine>(a, u, dg, key) : 0;
+            __syncthreads();
+            const int c = sm->hub[t];
+            __syncthreads();
+            return c;
+        } else {
+            sm->hub[t] = pos;
+            __syncthreads();
+            const int p = sm->hub[at];
+            if (any_long(u, dg)) long_children<Engine>(a, u, dg, key, p, dst, lab_base);
+            __syncthreads();
+            return 0;
         }
     }
 
@@ -593,8 +645,10 @@ struct Engine {
         const int T = blockDim.x;
         unsigned long long key = kKeyMax;
         int cnt = 0;
+        // (hubs apart: neighbours in the queue go to different warps)
+        const int mine = hubs() ? (int)(threadIdx.x & 31) * (T >> 5) + (int)(threadIdx.x >> 5) : (int)threadIdx.x;
         for (int i0 = lo; i0 < hi; i0 += T) {
-            const int i = i0 + (int)threadIdx.x;
+            const int i = i0 + mine;
             unsigned mask = 0;
             int r[8];
             int d = 0, u = -1;
@@ -1293,17 +1347,6 @@ struct Engine {
 
     // ---------------- labelled sweep (Alg. 3) ----------------
 
-    // A CTA's part of a level: cnt vertex ids, element j at sh[j] (shared memory) or g[step * j]
-    // (global: a staging buffer with step 1, or a label range of perm with step -1).
-    struct Slice {
-        const int* sh;
-        const int* g;
-        int step;
-        int cnt;
-    };
-
-    __device__ int sid(const Slice& s, int j) const { return s.sh ? s.sh[j] : ldcg(s.g + (long long)s.step * j); }
-
     __device__ Slice perm_range(int first, int cnt) const {
         Slice s;
         s.sh = nullptr;
@@ -1392,6 +1435,7 @@ struct Engine {
 
     // Phase A over a slice whose element j has key level_key(d, ord0 + j). Accumulates the min
     // (degree, id) over the slice. The round-0 row stays in (u0, r0) for phase B.
+    template <bool kHub = false>
     __device__ void phase_a(int d, unsigned long long ord0, const Slice& s, int& u0, int (&r0)[8],
                             bool with_key = true) {
         const int T = blockDim.x;
@@ -1424,7 +1468,8 @@ struct Engine {
                     }
                 }
             }
-            if (any_long(u, dg)) long_claims<Engine>(a, u, dg, key);
+            if constexpr (kHub) hub_round<kHubClaim>(d, ord0, s, j0, 0, nullptr, -1);
+            else if (any_long(u, dg)) long_claims<Engine>(a, u, dg, key);
         }
         if (with_key) accumulate(0, mk);
     }
@@ -1436,6 +1481,7 @@ struct Engine {
     // boff_base + j indexes this CTA's per-element offsets (disjoint between CTAs: the label of
     // element j minus the component's first label, or j in single-CTA runs).
     // Returns this CTA's child count and, in *out, the slice they form.
+    template <bool kHub = false>
     __device__ int phase_b(int d, unsigned long long ord0, const Slice& s, int u0, const int (&r0)[8],
                            int* ncache, int* stage, int* stail, int lab_base, int boff_base, Slice* out) {
         const int T = blockDim.x;
@@ -1467,7 +1513,8 @@ struct Engine {
                     u = -1;
                 }
             }
-            if (any_long(u, dg)) c += long_owned<Engine>(a, u, dg, key);
+            if constexpr (kHub) c += hub_round<kHubCount>(d, ord0, s, j0, 0, nullptr, -1);
+            else if (any_long(u, dg)) c += long_owned<Engine>(a, u, dg, key);
             int tot;
             const int ex = cta_scan(c, &tot);
             if (j0 == 0) {
@@ -1529,7 +1576,8 @@ struct Engine {
             }
             // the rest of a long row, in row order: a round's owned entries take consecutive
             // positions after the owner's earlier children
-            if (any_long(u, dg)) long_children<Engine>(a, u, dg, key, pos, dst, lab_base);
+            if constexpr (kHub) hub_round<kHubWrite>(d, ord0, s, j0, pos, dst, lab_base);
+            else if (any_long(u, dg)) long_children<Engine>(a, u, dg, key, pos, dst, lab_base);
         }
         __syncthreads();
         return carry;
@@ -1702,6 +1750,7 @@ struct Engine {
     // ownership; element j of CTA b's slice has order b * slot + j. Until the sweep ends (F = 0; d and the
     // prev_size vertices at prev_start are the last level), or the next level is small or out of balance: it
     // is then numbered (F vertices at lstart) and every CTA has seen it. Returns false on a failed wait.
+    template <bool kHub>
     __device__ bool grid_levels(int& d, int& lstart, int nv, Slice cur, int& prev_start, int& prev_size, int& F) {
         Ctl* c = a->ctl;
         const int b = cta_rank(), B = cta_count();
@@ -1723,7 +1772,7 @@ struct Engine {
                 publish_keys(d, ord0, cur);
                 round0_row(cur, u0, r0);
             } else {
-                phase_a(d, ord0, cur, u0, r0, false);
+                phase_a<kHub>(d, ord0, cur, u0, r0, false);
             }
             tick(kPhClaim);
             ExResult r;
@@ -1745,7 +1794,7 @@ struct Engine {
             if (b == 0 && threadIdx.x == 0) c->qtail[(d + 2) % 3] = 0;
             Slice nxt;
             int* stage = (d & 1) ? a->qa : a->qb;
-            const int kids = phase_b(d, ord0, cur, u0, r0, sm->cache[cb ^ 1], stage, &c->qtail[(d + 1) % 3], -1,
+            const int kids = phase_b<kHub>(d, ord0, cur, u0, r0, sm->cache[cb ^ 1], stage, &c->qtail[(d + 1) % 3], -1,
                                      lstart + r.pre - nv, &nxt);
             tick(kPhOwn);
             prev_start = lstart;
@@ -2028,7 +2077,8 @@ struct Engine {
             // ---- whole-grid levels ----
             if constexpr (!kCtaOnly) {
                 save_counters();
-                if (!run_grid_levels<kAsync, kBottomUp>(a, sm, d, lstart, nv, cur.g, cur.cnt, prev_start, prev_size))
+                if (!(hubs() ? run_grid_levels<kAsync, kBottomUp, true>(a, sm, d, lstart, nv, cur.g, cur.cnt, prev_start, prev_size)
+                             : run_grid_levels<kAsync, kBottomUp, false>(a, sm, d, lstart, nv, cur.g, cur.cnt, prev_start, prev_size)))
                     return false;
                 load_counters();
                 F = sm->wr.F;
@@ -2750,7 +2800,7 @@ __device__ __noinline__ bool run_grid_labelled(const EngineArgs* a, EngineSmem* 
     return true;
 }
 
-template <bool kAsync, bool kBottomUp>
+template <bool kAsync, bool kBottomUp, bool kHub>
 __device__ __noinline__ bool run_grid_levels(const EngineArgs* a, EngineSmem* sm, int d, int lstart, int nv,
                                              const int* g, int cnt, int prev_start, int prev_size) {
     Engine<false, false, kAsync, kBottomUp> e;
@@ -2763,7 +2813,7 @@ __device__ __noinline__ bool run_grid_levels(const EngineArgs* a, EngineSmem* sm
     cur.step = -1;
     cur.cnt = cnt;
     int F = 0;
-    if (!e.grid_levels(d, lstart, nv, cur, prev_start, prev_size, F)) return false;
+    if (!e.template grid_levels<kHub>(d, lstart, nv, cur, prev_start, prev_size, F)) return false;
     __syncthreads();
     if (threadIdx.x == 0) {
         sm->sw.prev_start = prev_start;

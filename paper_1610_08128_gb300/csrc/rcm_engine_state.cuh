@@ -13,8 +13,9 @@ constexpr int kWarpLevel = 32;  // narrow levels of at most this many vertices r
 // A level of a few hundred vertices that holds a hub is far more work than one CTA does quickly,
 // and a labelled first sweep over hubs costs more than a levels-only one: graphs with a vertex of
 // more than kHubDegree neighbours take a lower frontier switch and levels-only first sweeps by
-// default (the 1M-vertex power-law graph with hubs of 7,000: 24.3 ms with the grid defaults,
-// 8.8 ms with these).
+// default, and their whole-grid levels spread long rows over a CTA's warps (Engine::hub_round: a
+// 1M-vertex power-law graph with hubs of 7,000 entries 11.3 -> 6.2 ms a call; 24 ms with the grid's
+// defaults).
 constexpr int kHubDegree = 512;
 constexpr int kHubNarrow = 128;
 constexpr unsigned long long kClaimNone = ~0ull;
@@ -38,6 +39,8 @@ struct EngineArgs {
     int narrow_thr;
     int fused;
     int cc_first;                // persistent grid: build the component table before the first sweep
+    int hubs;                    // whole grid: the graph has a vertex of more than kHubDegree neighbours (set on
+                                 // the device)
     int hub_auto;                // default launch of the persistent grid: a graph with a vertex of more
                                  // than kHubDegree neighbours takes the frontier switch kHubNarrow and
                                  // levels-only first sweeps (decided on the device from ctl->maxdeg)
@@ -126,6 +129,7 @@ struct EngineSmem {
     unsigned long long xc_flag[2];  // (epoch << 32) | count, released at cluster scope
     unsigned long long xc_key[2];   // min (degree, id) key of the CTA's slice
     LocalState loc;
+    int* hub;                    // one int per thread: a round's values by element (Engine::hub_round)
     int cache[2][kCache];
 };
 

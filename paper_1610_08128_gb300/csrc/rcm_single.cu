@@ -489,6 +489,7 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
     args.obits = sl.obits > 0 ? sl.obits : claim_order_bits(n);
     args.profile = sl.profile;
     args.fused = sl.fused;
+    args.hubs = 0;
     args.hub_auto = sl.small ? 0 : sl.hub_auto;
     args.cc_first = sl.small ? 0 : sl.cc_first;
     args.limit_ns = sl.limit_ns;
