@@ -244,6 +244,7 @@ cudaError_t enqueue_batch(int G, long long n_total, int nnz, const long long* go
     Ctl* ctl = (Ctl*)(base + L.ctl);
     int* pool4 = (int*)(base + L.pool);
     int* deg = (int*)(base + L.deg);
+    unsigned char* deg8 = deg8_at(pool4, N);
     unsigned long long* claim = (unsigned long long*)(base + L.claim);
     int* vis = (int*)(base + L.vis);
     int* big = (int*)(base + L.big);
@@ -256,9 +257,9 @@ cudaError_t enqueue_batch(int G, long long n_total, int nnz, const long long* go
     // rows longer than small_max entries number at most nnz / (small_max + 1)
     const int big_grid = (int)std::max<long long>(1, std::min<long long>(3LL * di.sms, nnz / (t.small_max + 1)));
     // one pass over the entries checks the structure and each graph's block (G > 1) and counts degrees
-    k_degree_validate<<<pgrid, pb, 0, s>>>((int)n_total, nnz, rowptr, colidx, deg, claim, vis, big, ctl, t.small_max,
+    k_degree_validate<<<pgrid, pb, 0, s>>>((int)n_total, nnz, rowptr, colidx, deg, deg8, claim, vis, big, ctl, t.small_max,
                                            nullptr, nullptr, G > 1 ? goff : nullptr, G);
-    k_sort_rows_small<<<pgrid, pb, 0, s>>>((int)n_total, rowptr, colidx, deg, adj, ell, ctl, t.small_max,
+    k_sort_rows_small<<<pgrid, pb, 0, s>>>((int)n_total, rowptr, colidx, deg, deg8, adj, ell, ctl, t.small_max,
                                            t.by_degree);
     k_sort_rows_big<<<big_grid, kBigRowThreads, sizeof(unsigned long long) * kBigRowSmem, s>>>(
         (int)n_total, rowptr, colidx, deg, adj, ell, big, ctl, (unsigned long long*)pool4, t.by_degree);

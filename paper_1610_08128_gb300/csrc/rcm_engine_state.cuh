@@ -17,6 +17,11 @@ constexpr int kWarpLevel = 32;  // narrow levels of at most this many vertices r
 // 1M-vertex power-law graph with hubs of 7,000 entries 11.3 -> 6.2 ms a call; 24 ms with the grid's
 // defaults).
 constexpr int kHubDegree = 512;
+// Patterns this sparse likely fall into parts: 2-nearest-neighbour meshes and their spanning trees have
+// 2.7 neighbours a row, 3-nearest ones 3.7, grids 4 and 6. The probe sweep from the first start vertex runs
+// one part while everything else waits (1.2M-point mesh in 20 strips 9.6 -> 8.0 ms without it); the table
+// costs a pass of union-find, 0.3 ms per million vertices.
+constexpr int kPartsDegree = 32;
 constexpr int kHubNarrow = 128;
 constexpr unsigned long long kClaimNone = ~0ull;
 
@@ -38,7 +43,8 @@ struct EngineArgs {
     int* diag;                   // optional (may be null): first failed guard's site and value
     int narrow_thr;
     int fused;
-    int cc_first;                // persistent grid: build the component table before the first sweep
+    int cc_first;                // persistent grid: build the component table before the first sweep (-1: where
+                                 // the rows average fewer than kPartsDegree / 10 neighbours)
     int hubs;                    // whole grid: the graph has a vertex of more than kHubDegree neighbours (set on
                                  // the device)
     int hub_auto;                // default launch of the persistent grid: a graph with a vertex of more

@@ -14,13 +14,19 @@
 
 namespace rcm {
 
+constexpr int kDegLong = 64;  // longer rows are counted by the whole warp
+
 __global__ void k_degree_validate(int n, int nnz, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                                  int* __restrict__ deg, unsigned long long* __restrict__ claim, int* __restrict__ vis,
-                                  int* __restrict__ bigrows, Ctl* ctl, int small_max,
+                                  int* __restrict__ deg, unsigned char* __restrict__ deg8,
+                                  unsigned long long* __restrict__ claim, int* __restrict__ vis, int* __restrict__ bigrows, Ctl* ctl, int small_max,
                                   unsigned long long* __restrict__ adist, unsigned long long* __restrict__ fkey,
                                   const long long* __restrict__ goff, int G) {
     __shared__ int s_max;
-    if (threadIdx.x == 0) s_max = 0;
+    __shared__ unsigned long long s_sum;
+    if (threadIdx.x == 0) {
+        s_max = 0;
+        s_sum = 0;
+    }
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0 && (rowptr[0] != 0 || rowptr[n] != nnz || nnz < 0))
         atomicOr(&ctl->status, kErrBadCsr);
@@ -30,66 +36,115 @@ __global__ void k_degree_validate(int n, int nnz, const int* __restrict__ rowptr
         for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += stride)
             if (goff[g + 1] < goff[g]) atomicOr(&ctl->status, kErrBadCsr);
     }
-    // A warp takes 32 consecutive rows. In a batch, every entry of a row must stay inside its
-    // graph's block [goff[g], goff[g+1]): lane 0 finds the graph of the warp's first row (binary
-    // search) and every lane steps forward from there to its own.
+    // A CTA takes consecutive rows, a warp 32 at a time. In a batch, every entry of a row must stay inside
+    // its graph's block [goff[g], goff[g+1]): the warp finds the graph of its first row once (binary
+    // search), steps forward from there, and every lane steps on to its own. (Searched for every 32 rows,
+    // 14 dependent loads each, the 80M rows of 10,000 graphs took 1.09 ms here, so 0.65.)
     const int lane = threadIdx.x & 31;
     int local_max = 0;
-    for (int v0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); v0 < n; v0 += stride) {
+    unsigned local_sum = 0;  // at most the CTA's entries
+    const long long per = ((long long)n + gridDim.x - 1) / gridDim.x;
+    const int r0 = (int)min(per * blockIdx.x, (long long)n), r1 = (int)min(per * (blockIdx.x + 1), (long long)n);
+    int first = -1;  // graph of the warp's last 32 rows
+    for (int v0 = r0 + (int)(threadIdx.x & ~31u); v0 < r1; v0 += blockDim.x) {
         const int v = v0 + lane;
-        long long lo = 0, hi = n;
+        int lo = 0, hi = n;
         if (goff) {
-            int g = 0;
-            if (lane == 0) {
+            if (first < 0) {
                 int l = 0, h = G - 1;
                 while (l < h) {
                     const int mid = (l + h + 1) >> 1;
                     if (goff[mid] <= v0) l = mid; else h = mid - 1;
                 }
-                g = l;
+                first = l;
             }
-            g = __shfl_sync(0xffffffffu, g, 0);
-            if (v < n) {
+            while (first + 1 < G && goff[first + 1] <= v0) ++first;
+            if (v < r1) {
+                int g = first;
                 while (g + 1 < G && goff[g + 1] <= v) ++g;
-                lo = goff[g];
-                hi = goff[g + 1];
+                lo = (int)max(goff[g], 0LL);
+                hi = (int)min(goff[g + 1], (long long)n);
             }
         }
-        if (v >= n) continue;
-        const int a = rowptr[v], b = rowptr[v + 1];
-        int d = 0;
-        if (a < 0 || b < a || b > nnz) {
-            atomicOr(&ctl->status, kErrBadCsr);
-        } else {
-            for (int k = a; k < b; ++k) {
-                const int w = colidx[k];
-                if ((unsigned)w >= (unsigned)n || w < lo || w >= hi) {
-                    atomicOr(&ctl->status, kErrBadCsr);
-                } else if (w != v) {
-                    ++d;
+        int a = 0, b = 0, d = 0;
+        bool bad = false;
+        if (v < r1) {
+            a = rowptr[v];
+            b = rowptr[v + 1];
+            if (a < 0 || b < a || b > nnz) {
+                atomicOr(&ctl->status, kErrBadCsr);
+                a = b = 0;
+            }
+        }
+        // rows of more than kDegLong entries by the warp, one after another
+        for (unsigned m = __ballot_sync(0xffffffffu, b - a > kDegLong); m; m &= m - 1) {
+            const int src = __ffs(m) - 1, row = v0 + src;
+            const int ra = __shfl_sync(0xffffffffu, a, src), rb = __shfl_sync(0xffffffffu, b, src);
+            const int rlo = __shfl_sync(0xffffffffu, lo, src), rhi = __shfl_sync(0xffffffffu, hi, src);
+            int c = 0;
+            for (int k = ra + lane; k < rb; k += 32) {
+                const int w = __ldg(colidx + k);
+                bad |= w < rlo || w >= rhi;
+                c += w != row ? 1 : 0;
+            }
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == src) d = c;
+        }
+        if (v >= r1) {
+            if (bad) atomicOr(&ctl->status, kErrBadCsr);
+            continue;
+        }
+        {
+            // the others by their thread, 8 entries at a time, all loaded before the first is looked at
+            for (int k = a; k < b && b - a <= kDegLong; k += 8) {
+                int w[8];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) w[t] = k + t < b ? __ldg(colidx + k + t) : v;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    bad |= w[t] < lo || w[t] >= hi;
+                    d += w[t] != v ? 1 : 0;
                 }
             }
+            if (bad) atomicOr(&ctl->status, kErrBadCsr);
             if (b - a > small_max) bigrows[atomicAdd(&ctl->nbig, 1)] = v;
         }
         deg[v] = d;
+        deg8[v] = (unsigned char)min(d, kDeg8Many);
         claim[v] = ~0ull;
         vis[v] = 0;
         if (adist) adist[v] = ~0ull;
         if (fkey) fkey[v] = 0;
         local_max = max(local_max, d);
+        local_sum += (unsigned)d;
     }
-    atomicMax(&s_max, local_max);
+    __syncwarp();
+    local_max = __reduce_max_sync(0xffffffffu, local_max);
+    local_sum = __reduce_add_sync(0xffffffffu, local_sum);
+    if (lane == 0) {
+        atomicMax(&s_max, local_max);
+        atomicAdd(&s_sum, (unsigned long long)local_sum);
+    }
     __syncthreads();
-    if (threadIdx.x == 0) atomicMax(&ctl->maxdeg, s_max);
+    if (threadIdx.x == 0) {
+        atomicMax(&ctl->maxdeg, s_max);
+        atomicAdd(&ctl->degsum, s_sum);
+    }
 }
 
-// Rows of at most kSmallRowMax stored entries: one thread per row (sort_small_row).
+// Rows of at most kSmallRowMax stored entries: one thread per row (sort_small_row). Bound by the gathers of
+// the neighbours' degrees. A CTA takes consecutive rows, so in a batch the bytes it gathers are one graph's
+// at a time and stay in L1; with 4-byte degrees and rows dealt out in turn every gather was an L2 sector
+// (10,000 graphs, 80M rows: 1.88 -> 1.12 ms, with the one-word keys of sort_row8).
 __global__ void k_sort_rows_small(int n, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                                  const int* __restrict__ deg, int* __restrict__ adj, int4* __restrict__ ell,
-                                  const Ctl* ctl, int small_max, int by_degree) {
+                                  const int* __restrict__ deg, const unsigned char* __restrict__ deg8,
+                                  int* __restrict__ adj, int4* __restrict__ ell, const Ctl* ctl, int small_max,
+                                  int by_degree) {
     if (ctl->status & kErrBadCsr) return;
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
-        if (rowptr[v + 1] - rowptr[v] <= small_max) sort_small_row(v, rowptr, colidx, deg, adj, ell, by_degree);
+    const long long per = ((long long)n + gridDim.x - 1) / gridDim.x;
+    const int lo = (int)min(per * blockIdx.x, (long long)n), hi = (int)min(per * (blockIdx.x + 1), (long long)n);
+    for (int v = lo + (int)threadIdx.x; v < hi; v += blockDim.x)
+        if (rowptr[v + 1] - rowptr[v] <= small_max) sort_small_row(v, rowptr, colidx, deg, deg8, adj, ell, by_degree);
 }
 
 // Sorted row of v from keys[0, m) already sorted: the full row into adj (from offset a) and the

@@ -80,57 +80,83 @@ __device__ __forceinline__ unsigned long long row_key(const int* __restrict__ de
     return pack_key(by_degree ? __ldg(deg + w) : p, w);
 }
 
-__device__ __forceinline__ void cmp_swap(unsigned long long& x, unsigned long long& y) {
-    const unsigned long long lo = x < y ? x : y;
-    y = x < y ? y : x;
+template <class T>
+__device__ __forceinline__ void cmp_swap(T& x, T& y) {
+    const T lo = min(x, y);
+    y = max(x, y);
     x = lo;
 }
 
-// Rows of at most 8 stored entries (every row of the grids and meshes): keys in registers, sorted
-// by Batcher's 8-input odd-even merge network (19 compare-exchanges, no indexed local array).
-// Absent and diagonal entries get the largest key and sort to the end. Keys are unique, so the
-// order equals the insertion sort's.
-__device__ __forceinline__ void sort_row8(int v, int a, int len, const int* __restrict__ colidx,
-                                          const int* __restrict__ deg, int* __restrict__ adj,
-                                          int4* __restrict__ ell, int by_degree) {
-    unsigned long long k[8];
-    int m = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        k[i] = kKeyMax;
-        if (i < len) {
-            const int w = colidx[a + i];
-            if (w != v) {
-                k[i] = row_key(deg, w, i, by_degree);
-                ++m;
-            }
-        }
-    }
+// Batcher's 8-input odd-even merge network: 19 compare-exchanges, no indexed local array.
+template <class T>
+__device__ __forceinline__ void sort8(T (&k)[8]) {
     cmp_swap(k[0], k[1]); cmp_swap(k[2], k[3]); cmp_swap(k[4], k[5]); cmp_swap(k[6], k[7]);
     cmp_swap(k[0], k[2]); cmp_swap(k[1], k[3]); cmp_swap(k[4], k[6]); cmp_swap(k[5], k[7]);
     cmp_swap(k[1], k[2]); cmp_swap(k[5], k[6]);
     cmp_swap(k[0], k[4]); cmp_swap(k[1], k[5]); cmp_swap(k[2], k[6]); cmp_swap(k[3], k[7]);
     cmp_swap(k[2], k[4]); cmp_swap(k[3], k[5]);
     cmp_swap(k[1], k[2]); cmp_swap(k[3], k[4]); cmp_swap(k[5], k[6]);
-    int r[8];
+}
+
+// Degrees as bytes, for the row sorter's gathers: kDeg8Many stands for that many and more (looked up in
+// the full array). A sector holds 32 of them, so a graph's fit L1.
+constexpr int kDeg8Many = 255;
+constexpr int kNear = 1 << 23;  // ids this near their row's pack into 24 bits
+
+// Rows of at most 8 stored entries (every row of the grids and meshes), sorted in registers. Absent and
+// diagonal entries get the largest key and sort to the end. Keys are unique, so the order equals the
+// insertion sort's. Where every neighbour's id is near the row's and its degree a byte, a key is one word
+// (degree or position, then the id's distance) and a compare-exchange two instructions; otherwise 64 bits.
+__device__ __forceinline__ void sort_row8(int v, int a, int len, const int* __restrict__ colidx,
+                                          const int* __restrict__ deg, const unsigned char* __restrict__ deg8,
+                                          int* __restrict__ adj, int4* __restrict__ ell, int by_degree) {
+    int w[8];
 #pragma unroll
-    for (int i = 0; i < 7; ++i) r[i] = i < m ? (int)(unsigned)(k[i] & 0xffffffffu) : v;
-    r[7] = m;
-    store_ell(ell, v, r);
+    for (int i = 0; i < 8; ++i) w[i] = i < len ? __ldg(colidx + a + i) : v;
+    int d[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) d[i] = by_degree ? __ldg(deg8 + w[i]) : i;
+    unsigned k[8];
+    int m = 0;
+    bool near = true;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const unsigned off = (unsigned)w[i] - (unsigned)v + (unsigned)kNear;
+        const bool real = w[i] != v;
+        near &= !real || (off < 2u * kNear && d[i] != kDeg8Many);
+        k[i] = real ? (unsigned)d[i] << 24 | off : ~0u;
+        m += real ? 1 : 0;
+    }
+    int r[8];
+    if (near) {
+        sort8(k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) r[i] = i < m ? (int)(k[i] & 0xffffffu) - kNear + v : v;
+    } else {
+        unsigned long long kk[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) kk[i] = w[i] != v ? row_key(deg, w[i], i, by_degree) : kKeyMax;
+        sort8(kk);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) r[i] = i < m ? (int)(unsigned)(kk[i] & 0xffffffffu) : v;
+    }
     if (m > 7) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) adj[a + i] = (int)(unsigned)(k[i] & 0xffffffffu);
+        for (int i = 0; i < 8; ++i) adj[a + i] = r[i];
     }
+    r[7] = m;
+    store_ell(ell, v, r);
 }
 
 // Sorted row of a vertex with at most kSmallRowMax stored entries, by one thread: the padded row
 // and, for degree > 7, the full sorted row in adj (same offsets as the input row).
 __device__ __forceinline__ void sort_small_row(int v, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                                               const int* __restrict__ deg, int* __restrict__ adj,
+                                               const int* __restrict__ deg, const unsigned char* __restrict__ deg8,
+                                               int* __restrict__ adj,
                                                int4* __restrict__ ell, int by_degree) {
     const int a = rowptr[v], b = rowptr[v + 1];
     if (b - a <= 8) {
-        sort_row8(v, a, b - a, colidx, deg, adj, ell, by_degree);
+        sort_row8(v, a, b - a, colidx, deg, deg8, adj, ell, by_degree);
         return;
     }
     unsigned long long key[kSmallRowMax];
@@ -159,9 +185,12 @@ __device__ __forceinline__ void sort_small_row(int v, const int* __restrict__ ro
 // row is read beyond it. adist, fkey (may be null): the asynchronous sweeps' per-vertex words
 // (set to ~0) and the bottom-up frontier keys (set to 0). goff (may be null): a batch of G graphs
 // stacked block-diagonally; every row's entries must then stay inside its graph's block.
+// deg8: the degrees as bytes (kDeg8Many and above as kDeg8Many), for k_sort_rows_small; n bytes that nothing
+// else uses until then (deg8_at: the end of the frontier pool).
+inline unsigned char* deg8_at(int* pool4, long long n) { return (unsigned char*)(pool4 + 4 * n) - n; }
 __global__ void k_degree_validate(int n, int nnz, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                                  int* __restrict__ deg, unsigned long long* __restrict__ claim, int* __restrict__ vis,
-                                  int* __restrict__ bigrows, Ctl* ctl, int small_max,
+                                  int* __restrict__ deg, unsigned char* __restrict__ deg8,
+                                  unsigned long long* __restrict__ claim, int* __restrict__ vis, int* __restrict__ bigrows, Ctl* ctl, int small_max,
                                   unsigned long long* __restrict__ adist = nullptr,
                                   unsigned long long* __restrict__ fkey = nullptr,
                                   const long long* __restrict__ goff = nullptr, int G = 0);
@@ -170,8 +199,9 @@ __global__ void k_degree_validate(int n, int nnz, const int* __restrict__ rowptr
 // thread per row; k_degree_validate lists the longer ones for k_sort_rows_big with the same value.
 // by_degree: 1 = rows in (degree, id) order; 0 = stored order (the sort-free variant).
 __global__ void k_sort_rows_small(int n, const int* __restrict__ rowptr, const int* __restrict__ colidx,
-                                  const int* __restrict__ deg, int* __restrict__ adj, int4* __restrict__ ell,
-                                  const Ctl* ctl, int small_max, int by_degree = 1);
+                                  const int* __restrict__ deg, const unsigned char* __restrict__ deg8,
+                                  int* __restrict__ adj, int4* __restrict__ ell, const Ctl* ctl, int small_max,
+                                  int by_degree = 1);
 
 __global__ void k_sort_rows_big(int n, const int* __restrict__ rowptr, const int* __restrict__ colidx,
                                 const int* __restrict__ deg, int* __restrict__ adj, int4* __restrict__ ell,

@@ -312,7 +312,8 @@ rcm_status single_launch(int n, long long nnz, const rcm_options& o, SingleLaunc
     // hub graphs (a vertex of more than kHubDegree neighbours) take a lower switch and levels-only
     // first sweeps, decided on the device, when the caller left both at their defaults
     sl.hub_auto = o.narrow_threshold == 0 && o.fused_sweeps == 0 && !sl.async ? 1 : 0;
-    sl.cc_first = o.components_first > 0 ? 1 : 0;
+    // the component table before the first sweep: on request, or decided on the device (cc_auto)
+    sl.cc_first = o.components_first > 0 ? 1 : (o.components_first == 0 && !sl.cluster ? -1 : 0);
     sl.profile = o.profile_phases ? 1 : 0;
     sl.stall = o.debug_stall_barrier ? 1 : 0;
     sl.l2_persist = o.l2_persist > 0;
@@ -440,6 +441,7 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
     Ctl* ctl = (Ctl*)(base + L.ctl);
     int* pool4 = (int*)(base + L.pool4);
     int* deg = (int*)(base + L.deg);
+    unsigned char* deg8 = deg8_at(pool4, n);
     unsigned long long* claim = (unsigned long long*)(base + L.claim);
     int* vis = (int*)(base + L.vis);
     int* bigrows = (int*)(base + L.bigrows);
@@ -457,9 +459,9 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
     if (e == cudaSuccess) {
         const int pb = 256;
         const int pgrid = (int)std::min<long long>((n + pb - 1) / pb, (long long)di.sms * 16);
-        k_degree_validate<<<std::max(pgrid, 1), pb, 0, s>>>(n, (int)nnz, rowptr, colidx, deg, claim, vis, bigrows, ctl,
+        k_degree_validate<<<std::max(pgrid, 1), pb, 0, s>>>(n, (int)nnz, rowptr, colidx, deg, deg8, claim, vis, bigrows, ctl,
                                                            kSmallRowMax, adist, fkey);
-        k_sort_rows_small<<<std::max(pgrid, 1), pb, 0, s>>>(n, rowptr, colidx, deg, adj, ell, ctl, kSmallRowMax,
+        k_sort_rows_small<<<std::max(pgrid, 1), pb, 0, s>>>(n, rowptr, colidx, deg, deg8, adj, ell, ctl, kSmallRowMax,
                                                            sl.by_degree);
         // rows longer than kSmallRowMax entries number at most nnz / (kSmallRowMax + 1)
         const int big_grid = (int)std::max<long long>(1, std::min<long long>(3LL * di.sms, nnz / (kSmallRowMax + 1)));

@@ -93,7 +93,8 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
     int nv = Z;
     int C = -1;
     // with cc_first the component table is built before any sweep (no probe from the first start)
-    bool first = !args.cc_first, tried = false;
+    const bool parts = args.cc_first > 0 || (args.cc_first < 0 && __ldcg(&ctl->degsum) * 10 < (unsigned long long)n * kPartsDegree);
+    bool first = !parts, tried = false;
     while (nv < n) {
         if (!first && !tried && args.cc_cap > 0) {
             // more than one component: order them concurrently (one attempt)
