@@ -96,3 +96,12 @@ def test_components_of_one_graph(rcm, n):
         o.executor, o.components_first = 1, first
         got = rcm.order(device(g.rowptr), device(g.colidx), o).cpu().numpy()
         assert np.array_equal(got, oracle.rcm(g.n, g.rowptr, g.colidx)), first
+
+
+@pytest.mark.parametrize("npts", [45000, 50000, 400000])
+def test_many_components(rcm, npts):
+    """Raw 2-nearest-neighbour meshes: component tables around and well beyond one sort tile."""
+    g = synth.knn_mesh(npts, 2, npts)
+    got, stats = rcm.order(device(g.rowptr), device(g.colidx), with_stats=True)
+    assert stats["components"] > npts // 30
+    assert np.array_equal(got.cpu().numpy(), oracle.rcm(g.n, g.rowptr, g.colidx))
