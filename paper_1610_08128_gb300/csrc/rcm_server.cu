@@ -38,15 +38,15 @@
 
 namespace rcm {
 
-// Requests of at least this many vertices run on a cluster of kServeClusterBlocks CTAs by default
-// (see the header comment); the rest on one CTA of the batched executor. A cluster holds whole SMs
-// (one 512-thread CTA each) through levels that leave them mostly idle, while a single CTA takes a
-// third of an SM: on GB300, ordering a 1M-vertex 2D grid took 18 ms on a cluster of 6 and 32 ms on
-// one CTA, about ten times the SM time. So clusters pay off only for the largest requests, whose
-// latency they cut most. Measured on the 2,000 req/s trace (4,000 requests, pool of 256):
-// clusters of 4 from 512k vertices 1,863/s, p50 27 ms, p99 159 ms; clusters of 6 from 256k
-// vertices 1,789/s, 60 / 205 ms; no clusters 1,103/s, 688 / 1,519 ms.
-constexpr long long kServeClusterMin = 1LL << 19;
+// Requests of at least kServeClusterMin vertices run on a cluster by default, smaller ones on one CTA. With
+// the one CTA's state in shared memory it orders up to a million vertices in half the SM time a cluster
+// needs. The cluster has kServeClusterBlocks CTAs under load and kServeClusterIdle while at most
+// kServeFew requests are in the server (they would leave SMs idle). GB300, 48 requests of 1,000 to 4M
+// vertices at once: 102 ms with clusters of 4 from 524,288 vertices, 90 from 1,048,576, 75 with 8 CTAs
+// there; 800 requests at once (32 hardware queues, 256 in flight): 1,680, 2,702 and 1,838 orderings/s.
+constexpr int kServeClusterIdle = 8;
+constexpr int kServeFew = 64;
+constexpr long long kServeClusterMin = 1LL << 20;
 constexpr int kServeClusterBlocks = 4;
 
 // Arena bytes of one request: the staged CSR and result when they are in host memory, a 256-byte
@@ -132,6 +132,7 @@ struct Request {
     size_t off = 0, bytes = 0;
     int slot = -1;
     int state = 0;  // 0 waiting, 1 running, 2 done
+    bool few = false;     // admitted while the server held few requests
     bool orphan = false;  // finished by the failure path: its host function may still be pending
     rcm_status status = RCM_OK;
     double t_submit = 0, t_start = 0, t_done = 0;
@@ -167,7 +168,7 @@ struct Server {
     int running = 0, max_running = 0;
     cudaError_t broken = cudaSuccess;  // first stream error seen: the context is unusable
     long long cluster_min = kServeClusterMin;  // -1: never
-    int cluster_blocks = kServeClusterBlocks;
+    int cluster_blocks = 0;                    // 0: by load
     int debug_fail_after = 0;                  // test hook (rcm_server_options)
     bool trace = false;                // RCM_TRACE_ERRORS set: failed requests are reported on stderr
 };
@@ -264,7 +265,8 @@ static rcm_status launch_request(Server* s, Request* r) {
         const SingleLayout L = single_layout(r->n, r->nnz);
         rcm_options o{};
         o.cluster = 1;
-        o.grid_blocks = s->cluster_blocks;
+        o.grid_blocks = s->cluster_blocks ? s->cluster_blocks
+                        : r->few ? std::min(kServeClusterIdle, single_cluster_max()) : kServeClusterBlocks;
         SingleLaunch sl;
         const rcm_status ls = single_launch(r->n, r->nnz, o, &sl);
         if (ls != RCM_OK) return ls;
@@ -357,6 +359,7 @@ static void worker_loop(Server* s) {
             r->t_start = now_s();
             s->running++;
             s->max_running = std::max(s->max_running, s->running);
+            r->few = s->running + (int)s->waiting.size() <= kServeFew;
             admit.push_back(r);
         }
         if (!admit.empty()) {
@@ -444,7 +447,7 @@ rcm_status rcm_server_create_ex(size_t hbm_budget_bytes, int32_t max_inflight, c
     s.max_inflight = max_inflight;
     if (opts) {
         s.cluster_min = opts->cluster_min_vertices == 0 ? kServeClusterMin : opts->cluster_min_vertices;
-        s.cluster_blocks = opts->cluster_blocks == 0 ? kServeClusterBlocks : opts->cluster_blocks;
+        s.cluster_blocks = opts->cluster_blocks;
         s.debug_fail_after = opts->debug_fail_after;
     }
     s.slot_req.assign(max_inflight, nullptr);
