@@ -156,7 +156,9 @@ template <int kThreads, bool kAsync, bool kBottomUp>
 __global__ void __launch_bounds__(kThreads, 1) k_rcm_single(EngineArgs args, int stall) {
     __shared__ EngineSmem smem;
     __shared__ int s_item;
-    extern __shared__ unsigned long long s_sort[];  // component-table sort (kCompSmem entries)
+    // component-table sort (kCompSmem entries), on CTA 0 also the local sweeps' state, whose bitmap is
+    // read 16 bytes at a time: without the attribute the array starts wherever the static part ends
+    extern __shared__ __align__(16) unsigned long long s_sort[];
     // launched in clusters for the middle tier: every CTA's exchange words are cleared before any
     // peer can read them, and no CTA leaves while a peer may still read its shared memory (every
     // path of single_run ends: all its waits are bounded)
