@@ -161,8 +161,9 @@ typedef struct {
                                   sweep does not reach every vertex. Faster on graphs known to be
                                   disconnected into components of similar size (that probe sweep is
                                   serial); one union-find pass more on a connected graph. Same
-                                  result. -1 = off; 0 = where the rows average fewer than 3.2
-                                  neighbours (decided on the device; off on a cluster)              */
+                                  result. -1 = off; 0 = decided on the device: where the rows average
+                                  fewer than 3.2 neighbours that first sweep gives up for the table
+                                  if its 64th level is narrow (off on a cluster)                    */
 } rcm_options;
 
 /* Statistics of one ordering (filled by rcm_order_ex when requested). */

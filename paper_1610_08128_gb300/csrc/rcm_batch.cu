@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(kThreads, batch_min_blocks<kThreads>()) k_rcm_
         a.cc_big = 0;
         a.fused = 1;
         a.hubs = 0;
+        a.probe = 0;
         a.hub_auto = 0;
         a.cc_first = 0;
         a.limit_ns = 0;

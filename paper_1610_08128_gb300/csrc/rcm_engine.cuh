@@ -1192,10 +1192,11 @@ struct Engine {
     }
 
     // Levels-only sweep from root. On return: ecc, the min (degree, id) key of the last level and
-    // the number of vertices reached (the component's size).
+    // the number of vertices reached (the component's size). With a->probe set (whole grid) the sweep gives
+    // up with ecc = -1 where that level is still narrow (see component).
     __device__ bool sweep_levels(int root, int& ecc, unsigned long long& last_key, long long& reached) {
         if constexpr (kAsync) {
-            if (a->adist && async_ok) {
+            if (a->adist && async_ok && a->probe == 0) {
                 const int rc = sweep_async(root, ecc, last_key, reached);
                 if (rc >= 0) return rc == 1;
                 async_ok = false;  // the queue ran full: this and later sweeps run level by level
@@ -1226,6 +1227,7 @@ struct Engine {
             if (kCtaOnly || F < a->narrow_thr) {
                 unsigned long long lk = kKeyMax;
                 if (kCtaOnly || b == 0) {
+                    const int stop = !kCtaOnly && a->probe > ecc ? a->probe : kIntMax;
                     if (!in_cache) {
                         for (int i = threadIdx.x; i < F; i += blockDim.x) sm->cache[cb][i] = ldcg(cur + i);
                         in_cache = true;
@@ -1279,7 +1281,7 @@ struct Engine {
                             fail_at(kSiteLevels, ecc);
                             return false;
                         }
-                        if (!kCtaOnly && F >= a->narrow_thr) break;
+                        if (!kCtaOnly && (F >= a->narrow_thr || ecc >= stop)) break;
                     }
                     if (kCtaOnly) {
                         __syncthreads();
@@ -1288,7 +1290,7 @@ struct Engine {
                     }
                     if (threadIdx.x == 0) {
                         c->pub_F = F;
-                        c->pub_cur = (cur == a->qb) ? 1 : 0;
+                        c->pub_cur = (cur == a->qb ? 1 : 0) | (F > 0 && ecc >= stop ? 2 : 0);
                         c->pub_ecc = ecc;
                         c->pub_key = lk;
                         c->pub_reached = reached;
@@ -1310,11 +1312,15 @@ struct Engine {
                 lk = sm->bck;
                 reached = __ldcg(&c->pub_reached);
                 __syncthreads();
-                cur = pc ? a->qb : a->qa;
-                nxt = pc ? a->qa : a->qb;
+                cur = (pc & 1) ? a->qb : a->qa;
+                nxt = (pc & 1) ? a->qa : a->qb;
                 in_cache = false;
                 if (Fp == 0) {
                     last_key = lk;
+                    return true;
+                }
+                if (pc & 2) {
+                    ecc = -1;
                     return true;
                 }
                 F = Fp;
@@ -1823,7 +1829,8 @@ struct Engine {
     }
 
     // Labelled sweep from root, labels from nv. On return: ecc, the min (degree, id) key of the
-    // last level, and the component size (labels nv .. nv+size-1).
+    // last level, and the component size (labels nv .. nv+size-1). With a->probe set (whole grid) the sweep
+    // gives up with ecc = -1 and size the vertices numbered so far where that level is still narrow.
     __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size) {
         Ctl* c = a->ctl;
         const int b = cta_rank(), B = cta_count();
@@ -1856,6 +1863,7 @@ struct Engine {
                 int lastF = 0;
                 const int from = lstart + F;  // first label of the run's first new level
                 if (kCtaOnly || b == 0) {
+                    const int stop = !kCtaOnly && a->probe > d ? a->probe : kIntMax;
                     if (grid_local()) {
                         local_run<false>(a, sm, lstart == nv, d, lstart, F, a->local_hi);
                         if (sm->wr.bad) {
@@ -1923,7 +1931,7 @@ struct Engine {
                             fail_at(kSiteLevels, d);
                             return false;
                         }
-                        if (!kCtaOnly && F >= a->narrow_thr) break;
+                        if (!kCtaOnly && (F >= a->narrow_thr || d >= stop)) break;
                     }
                     if (kCtaOnly) {
                         last_key = lk;
@@ -1936,7 +1944,7 @@ struct Engine {
                         c->pub_start = lstart;
                         c->pub_ecc = d;
                         c->pub_key = lk;
-                        c->pub_lastF = lastF;
+                        c->pub_lastF = F > 0 && d >= stop ? -1 : lastF;
                         c->pub_reached = from;
                         c->qtail[0] = c->qtail[1] = c->qtail[2] = 0;
                     }
@@ -1962,6 +1970,11 @@ struct Engine {
                     last_key = lk;
                     ecc = d;
                     size = lstart + lastF2 - nv;
+                    return true;
+                }
+                if (lastF2 < 0) {  // gave up
+                    ecc = -1;
+                    size = lstart + F - nv;
                     return true;
                 }
                 if (grid_local()) {
@@ -2277,7 +2290,8 @@ struct Engine {
     // all_left >= 0 (the number of vertices not yet numbered), the call stops after the first
     // sweep when the component is smaller than that, is small enough for the component table to
     // order it at least as fast, and holds less than 3/4 of the vertices left, returning
-    // size = -1 (nothing numbered).
+    // size = -1 (nothing numbered). With a->probe set it also stops where that level of the sweep is still
+    // narrow (on the whole grid): size = minus the vertices reached by then.
     __device__ bool component(int r, int nv, int& size, long long all_left = -1) {
         if (!in_graph(r) || nv < 0 || nv >= a->n) {
             fail_at(kSiteStart, r);
@@ -2298,6 +2312,14 @@ struct Engine {
             tick(kPhOther);
         } else if (!levels(r, ecc_prev, k1, reached)) {
             return false;
+        }
+        if constexpr (!kCtaOnly) {
+            if (threadIdx.x == 0) sm->args.probe = 0;  // (every sweep ends with a barrier)
+            __syncthreads();
+            if (ecc_prev < 0) {  // gave up
+                size = -(int)reached;
+                return true;
+            }
         }
         // The start vertex's component does not hold every vertex left: the others get a component
         // table. The component is finished here, its sweep kept, when the table would order it no

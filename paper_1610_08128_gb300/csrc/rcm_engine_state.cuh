@@ -17,11 +17,22 @@ constexpr int kWarpLevel = 32;  // narrow levels of at most this many vertices r
 // 1M-vertex power-law graph with hubs of 7,000 entries 11.3 -> 6.2 ms a call; 24 ms with the grid's
 // defaults).
 constexpr int kHubDegree = 512;
-// Patterns this sparse likely fall into parts: 2-nearest-neighbour meshes and their spanning trees have
+// Patterns this sparse may fall into parts: 2-nearest-neighbour meshes and their spanning trees have
 // 2.7 neighbours a row, 3-nearest ones 3.7, grids 4 and 6. The probe sweep from the first start vertex runs
-// one part while everything else waits (1.2M-point mesh in 20 strips 9.6 -> 8.0 ms without it); the table
-// costs a pass of union-find, 0.3 ms per million vertices.
+// one part while everything else waits (1.2M-point mesh in 20 strips 9.6 ms with it, 8.0 without); the
+// component table costs a pass of union-find, 0.3 ms per million vertices. Trees, cubic and other sparse random
+// graphs are as sparse, but connected and low, and the table is lost on them. So the probe runs, and gives
+// up for the table where level kProbeLevels is still narrow (0.1 ms of the strips' 8.0; a 20,000-vertex tree
+// 0.64 ms, and 0.94 with 32 levels, where it gives up).
 constexpr int kPartsDegree = 32;
+constexpr int kProbeLevels = 64;
+// Levels of up to this many vertices are one CTA's work: a 50,000-vertex path 72 ms on 256 threads, 84 on
+// CTA 0 of the grid; a 260^2 grid with its edges halved 5.6 and 5.1.
+constexpr int kThinLevel = 8;
+// Of a component table the grid keeps what holds 3/4 of the vertices left, from this size on (below it one
+// CTA is the faster, as for whole graphs): a cubic graph of 200,000 vertices 0.28 ms on the grid, 14.8 on one
+// CTA, a random tree 1.0 and 26, the giant component of a sparse random graph 1.1 and 39.
+constexpr int kGridMin = 4609;
 constexpr int kHubNarrow = 128;
 constexpr unsigned long long kClaimNone = ~0ull;
 
@@ -44,7 +55,7 @@ struct EngineArgs {
     int narrow_thr;
     int fused;
     int cc_first;                // persistent grid: build the component table before the first sweep (-1: where
-                                 // the rows average fewer than kPartsDegree / 10 neighbours)
+                                 // the rows average fewer than kPartsDegree / 10 neighbours and the probe gives up)
     int hubs;                    // whole grid: the graph has a vertex of more than kHubDegree neighbours (set on
                                  // the device)
     int hub_auto;                // default launch of the persistent grid: a graph with a vertex of more
@@ -82,6 +93,8 @@ struct EngineArgs {
     int local_hi;                // a run ends at a level of this many vertices (narrow_thr starts one)
     int local_slots, local_entries;
     unsigned* gvis;              // bitmap of n vertices: what the grid's levels visited, for the next run
+    int probe;                   // whole grid: a level at which a sweep that is still narrow gives up (0 = none; set
+                                 // on the device)
 };
 
 enum { kPhExpand = 0, kPhClaim, kPhOwn, kPhLabels, kPhExchange, kPhRedist, kPhWaitNarrow, kPhOther };

@@ -59,6 +59,7 @@ struct alignas(128) Ctl {
     int pub_lastF;   // size of the last non-empty level when finished
     int comp_count;  // component-table entries left to k_rcm_components (0 = none)
     int comp_nv;     // first label those components may take
+    int comp_big;    // entries of at least this many vertices were ordered by the whole grid
     int cc_open;     // vertices still unnumbered when the component table is built
     unsigned long long degsum;     // off-diagonal entries
     unsigned long long pub_key;    // min (degree, id) key of the last level when finished

@@ -760,10 +760,11 @@ struct Local {
     }
 
     // Labelled levels from level d of F vertices at labels lstart.., held in cache buffer cb, until one is
-    // the last (returns true: F and lstart are its) or the next has at least `hi` vertices (returns false:
-    // they are the next one's). `bad` is set where a label left the graph.
-    __device__ bool labelled_levels(int& F, int& lstart, int& cb, int& d, int hi, bool& bad) {
+    // the last (returns true: F and lstart are its) or the next has at least `hi` vertices or is level
+    // `stop` (returns false: they are the next one's). `bad` is set where a label left the graph.
+    __device__ bool labelled_levels(int& F, int& lstart, int& cb, int& d, int hi, int stop, bool& bad) {
         const unsigned c0 = s_addr(sm->cache[0]);
+        int left = stop - d;  // counted down in place of a level number
         while (true) {
             next_generation();
             int kids = labelled_level(F, lstart, c0 + 4 * kCache * cb, c0 + 4 * kCache * (cb ^ 1), bad);
@@ -772,12 +773,17 @@ struct Local {
                 kids = local_wide_level<kDirect>(a, sm, F, lstart, cb, gen, seq);
                 bad |= kids < 0;
             }
-            if (kids <= 0) return true;
+            if (kids <= 0) {
+                d = stop - left;
+                return true;
+            }
             lstart += F;
             F = kids;
             cb ^= 1;
-            ++d;
-            if (F >= hi) return false;
+            if (--left == 0 || F >= hi) {
+                d = stop - left;
+                return false;
+            }
         }
     }
 
@@ -797,7 +803,7 @@ struct Local {
         int F = 1, cb = 0, lstart = nv;
         bool bad = false;
         ecc = 0;
-        labelled_levels(F, lstart, cb, ecc, kIntMax, bad);
+        labelled_levels(F, lstart, cb, ecc, kIntMax, kIntMax, bad);
         last_key = labelled_key(F, lstart, cb);
         size = lstart + F - nv;
         return !__syncthreads_or(bad);
@@ -805,7 +811,8 @@ struct Local {
 
     // A run of narrow levels on CTA 0 of the grid: level d, F (below kCache) vertices at labels lstart..
     // in perm. first: the sweep starts here, nothing else is visited; otherwise gvis holds what the grid's
-    // levels visited since the last run. Runs until the sweep ends or a level has `hi` vertices.
+    // levels visited since the last run. Runs until the sweep ends, a level has `hi` vertices or, where
+    // a->probe is set and not yet passed, that level is next.
     __device__ void run(bool first, int d, int lstart, int F, int hi) {
         const int words = local_vis_words(n) / 4;
         uint4* v = (uint4*)sm->loc.vis;
@@ -832,7 +839,7 @@ struct Local {
         const int d0 = d;
         int cb = 0;
         bool bad = false;
-        const bool end = labelled_levels(F, lstart, cb, d, hi, bad);
+        const bool end = labelled_levels(F, lstart, cb, d, hi, a->probe > d ? a->probe : kIntMax, bad);
         const unsigned long long key = end ? labelled_key(F, lstart, cb) : kKeyMax;
         bad = __syncthreads_or(bad);
         save();

@@ -312,7 +312,7 @@ rcm_status single_launch(int n, long long nnz, const rcm_options& o, SingleLaunc
     // hub graphs (a vertex of more than kHubDegree neighbours) take a lower switch and levels-only
     // first sweeps, decided on the device, when the caller left both at their defaults
     sl.hub_auto = o.narrow_threshold == 0 && o.fused_sweeps == 0 && !sl.async ? 1 : 0;
-    // the component table before the first sweep: on request, or decided on the device (cc_auto)
+    // the component table before the first sweep: on request, or decided on the device (-1)
     sl.cc_first = o.components_first > 0 ? 1 : (o.components_first == 0 && !sl.cluster ? -1 : 0);
     sl.profile = o.profile_phases ? 1 : 0;
     sl.stall = o.debug_stall_barrier ? 1 : 0;
@@ -492,6 +492,7 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
     args.profile = sl.profile;
     args.fused = sl.fused;
     args.hubs = 0;
+    args.probe = 0;
     args.hub_auto = sl.small ? 0 : sl.hub_auto;
     args.cc_first = sl.small ? 0 : sl.cc_first;
     args.limit_ns = sl.limit_ns;

@@ -91,10 +91,15 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
     e.stat_add(kStIsolated, Z);
     e.stat_add(kStComponents, Z);
     int nv = Z;
-    int C = -1;
-    // with cc_first the component table is built before any sweep (no probe from the first start)
-    const bool parts = args.cc_first > 0 || (args.cc_first < 0 && __ldcg(&ctl->degsum) * 10 < (unsigned long long)n * kPartsDegree);
-    bool first = !parts, tried = false;
+    int C = -1, big = args.cc_big;
+    // with cc_first the component table is built before any sweep (no probe from the first start); where
+    // the pattern only looks like several parts, a probe decides, which gives up while it is cheap
+    const bool sparse = __ldcg(&ctl->degsum) * 10 < (unsigned long long)n * kPartsDegree;
+    bool first = args.cc_first <= 0, tried = false, thin = false;
+    if (args.cc_first < 0 && sparse && args.cc_cap > 0) {
+        if (threadIdx.x == 0) smem.args.probe = kProbeLevels;
+        __syncthreads();
+    }
     while (nv < n) {
         if (!first && !tried && args.cc_cap > 0) {
             // more than one component: order them concurrently (one attempt)
@@ -102,7 +107,13 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
             C = e.cc_prepare(nv, s_sort, kCompSmem);
             if (C == -2) return;
             if (threadIdx.x == 0) smem.loc.gen = ~0u;  // the sort used the local sweeps' memory
-            if (C > 0) break;
+            if (C > 0) {
+                // nothing runs beside a component that holds most of what is left: it keeps the grid, unless
+                // the probe saw it (its start vertex is the first) to be so thin that one CTA is the faster
+                const int most = max((int)((3LL * (n - nv) + 3) / 4), kGridMin);
+                if (!thin || __ldcg(&args.cc_tab[0].z) < most) big = min(big, most);
+                break;
+            }
         }
         unsigned long long k0;
         if (!e.next_start(k0)) return;
@@ -115,7 +126,10 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
         const long long left = (first && args.cc_cap > 0) ? (long long)(n - nv) : -1;
         first = false;
         if (!e.component((int)(unsigned)(k0 & 0xffffffffu), nv, size, left)) return;
-        if (size < 0) continue;  // more components: the next iteration prepares them all
+        if (size < 0) {  // more components, or a long one: the next iteration prepares them all
+            thin = size < -1 && -size <= kProbeLevels * kThinLevel;
+            continue;
+        }
         // runs of local levels leave no claims: the vertices just numbered are marked for the searches
         if (e.grid_local() && nv + size < n && !e.mark_labels(nv, size)) return;
         nv += size;
@@ -128,7 +142,7 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
                 e.fail_at(kSiteTable, i);
                 return;
             }
-            if (t.z < args.cc_big) continue;
+            if (t.z < big) continue;
             int size;
             if (!e.component(t.x, t.y, size)) return;
             if (size != t.z) {
@@ -149,6 +163,7 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
     if (C > 0 && blockIdx.x == 0 && threadIdx.x == 0) {
         ctl->comp_count = C;
         ctl->comp_nv = nv;
+        ctl->comp_big = big;
     }
 }
 
@@ -184,7 +199,7 @@ __global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args, in
     __shared__ int s_item;
     Ctl* ctl = args.ctl;
     if (ld_volatile(&ctl->status) & (kErrBadCsr | kErrInternal | kErrTimeout | kErrTooLarge)) return;
-    const int C = ctl->comp_count, nv = ctl->comp_nv;  // written by the previous kernel on this stream
+    const int C = ctl->comp_count, nv = ctl->comp_nv, big = ctl->comp_big;  // written by the previous kernel on this stream
     if (C <= 0) return;
     Engine<true, false, false, false, true> e;
     EngineArgs first = args;
@@ -197,7 +212,7 @@ __global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args, in
     // tiny components, one per thread of the grid, all at once
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < C; i += gridDim.x * blockDim.x) {
         const int4 t = __ldcg(args.cc_tab + i);
-        if (t.z > kTinyMax || t.z >= args.cc_big) continue;
+        if (t.z > kTinyMax || t.z >= big) continue;
         if (!e.tab_ok(t, nv)) {
             e.fail_at(kSiteTable, i);
             break;
@@ -213,7 +228,7 @@ __global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args, in
         __syncthreads();
         if (i >= C) break;
         const int4 t = __ldcg(args.cc_tab + i);
-        if (t.z >= args.cc_big || t.z <= kTinyMax) continue;
+        if (t.z >= big || t.z <= kTinyMax) continue;
         if (!e.tab_ok(t, nv)) {
             e.fail_at(kSiteTable, i);
             return;
