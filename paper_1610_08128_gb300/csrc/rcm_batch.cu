@@ -17,9 +17,11 @@ namespace rcm {
 
 // The local sweeps' lists take levels of about a thousand vertices. The table takes the shared memory
 // that is left, up to kBatchSlots: the emptier it is, the fewer probes (levels of 500 vertices on 512
-// threads: claims 2,500 -> 1,650 cycles with 8,192 slots instead of 2,048).
+// threads: claims 2,500 -> 1,650 cycles with 8,192 slots instead of 2,048), but what it takes is L1 that
+// wider levels, in global memory, read their rows through (twenty graphs of up to 839,000 vertices, 3D grids
+// among them: 31.8 ms with 8,192, 19.2 with 4,096, 17.1 with 2,048; a 900,000-point mesh 30.5, 30.6 and 32.1).
 constexpr int kBatchEntries = 3072;
-constexpr int kBatchSlots = 8192;
+constexpr int kBatchSlots = 4096;
 constexpr int kBatchMinSlots = 2048;
 constexpr int kBatchStaticSmem = 18 * 1024;  // EngineSmem and the rest, rounded up
 constexpr int kSmemPerSm = 227 * 1024;

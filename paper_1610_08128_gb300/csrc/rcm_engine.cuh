@@ -105,6 +105,11 @@ template <bool kAsync, bool kBottomUp, bool kHub>
 __device__ __noinline__ bool run_grid_levels(const EngineArgs* a, EngineSmem* sm, int d, int lstart, int nv,
                                              const int* g, int cnt, int prev_start, int prev_size);
 
+// The rest of a CTA engine's labelled sweep from level d on, F vertices at labels from lstart, in global
+// memory (out of line for the same reason). Results in sm->sw.
+template <bool kWarp>
+__device__ __noinline__ bool run_wide_rest(const EngineArgs* a, EngineSmem* sm, int root, int nv, int d, int lstart, int F);
+
 template <bool kCtaOnly, bool kSmem = false, bool kAsync = false, bool kBottomUp = false, bool kWarp = kSmem>
 struct Engine {
     static_assert(kCtaOnly || !kSmem, "shared-memory state needs a CTA engine");
@@ -1831,7 +1836,10 @@ struct Engine {
     // Labelled sweep from root, labels from nv. On return: ecc, the min (degree, id) key of the
     // last level, and the component size (labels nv .. nv+size-1). With a->probe set (whole grid) the sweep
     // gives up with ecc = -1 and size the vertices numbered so far where that level is still narrow.
-    __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size) {
+    // F0 > 0 (CTA engines): the sweep goes on at level d0, F0 vertices at labels from lstart0, with the
+    // vertices numbered so far marked.
+    __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size, int d0 = 0,
+                                   int lstart0 = 0, int F0 = 0) {
         Ctl* c = a->ctl;
         const int b = cta_rank(), B = cta_count();
         const unsigned long long slot = kCtaOnly ? 0ull : ((1ull << a->obits) - 1ull) / (unsigned long long)B;
@@ -1857,6 +1865,12 @@ struct Engine {
         // the last completed level (grid runs detect the end one level late)
         int prev_start = nv, prev_size = 1;
         int known = nv;     // labels below this are in CTA 0's bitmap (grid_local)
+        if (kCtaOnly && F0 > 0) {
+            d = d0;
+            lstart = lstart0;
+            F = F0;
+            cur = perm_range(lstart, F);
+        }
         while (true) {
             if (narrow) {
                 unsigned long long lk = kKeyMax;
@@ -2146,6 +2160,9 @@ struct Engine {
         return false;
     }
 
+    // Whether the last labelled sweep left claims in global memory.
+    __device__ bool claimed() const { return !local() || sm->loc.rest > 0; }
+
     // The engine's counters (the same in every thread) handed to an out-of-line sweep and taken back.
     __device__ void save_counters() {
         if (threadIdx.x == 0) {
@@ -2200,10 +2217,25 @@ struct Engine {
                 last_key = sm->wr.lk;
                 size = (int)sm->wr.reached;
                 tick(kPhOwn);
-                stat_add(kStNarrow, ecc + 1);
                 if (sm->wr.bad) {
                     fail(kErrInternal);
                     return false;
+                }
+                const int rest = sm->loc.rest;
+                stat_add(kStNarrow, rest > 0 ? ecc : ecc + 1);
+                if constexpr (!kSmem) {
+                    if (rest > 0) {
+                        // a level too wide for the lists or the table, and the next ones likely too: the
+                        // rest of the sweep in global memory
+                        mark_labels(nv, size);
+                        save_counters();
+                        if (!run_wide_rest<kWarp>(a, sm, root, nv, ecc, nv + size - rest, rest)) return false;
+                        load_counters();
+                        ecc = sm->sw.ecc;
+                        last_key = sm->sw.key;
+                        size = sm->sw.size;
+                        __syncthreads();
+                    }
                 }
                 return true;
             }
@@ -2308,7 +2340,7 @@ struct Engine {
             if (!labelled(r, nv, ecc_prev, k1, sz)) return false;
             reached = sz;
             tick(kPhOther);
-            if (!local() && !reset_claims(nv, sz)) return false;
+            if (claimed() && !reset_claims(nv, sz)) return false;
             tick(kPhOther);
         } else if (!levels(r, ecc_prev, k1, reached)) {
             return false;
@@ -2352,7 +2384,7 @@ struct Engine {
                 }
                 ecc_prev = ecc;
                 tick(kPhOther);
-                if (!local() && !reset_claims(nv, size)) return false;
+                if (claimed() && !reset_claims(nv, size)) return false;
                 tick(kPhOther);
                 r = (int)(unsigned)(k2 & 0xffffffffu);
             }
@@ -2856,6 +2888,25 @@ __device__ __noinline__ void long_children(const EngineArgs* a, int u, int dg, u
         }
         pos += __popc(bal & mine);
     });
+}
+
+template <bool kWarp>
+__device__ __noinline__ bool run_wide_rest(const EngineArgs* a, EngineSmem* sm, int root, int nv, int d, int lstart, int F) {
+    Engine<true, false, false, false, kWarp> e;
+    e.a = a;
+    e.sm = sm;
+    e.load_counters();
+    int ecc, size;
+    unsigned long long key;
+    if (!e.sweep_labelled(root, nv, ecc, key, size, d, lstart, F)) return false;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sm->sw.ecc = ecc;
+        sm->sw.key = key;
+        sm->sw.size = size;
+    }
+    e.save_counters();
+    return true;
 }
 
 template <bool kAsync, bool kBottomUp>

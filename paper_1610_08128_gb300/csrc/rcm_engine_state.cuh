@@ -109,6 +109,7 @@ struct LocalState {
     unsigned* hval;      // ((gmax - generation) << idbits) | smallest frontier position
     unsigned gen;        // generation of the last labelled level
     unsigned seq;        // labelled sweeps so far (tags the global claims)
+    int rest;            // vertices of the level at which the last sweep went on in global memory (0 = it did not)
     unsigned* list;      // the warps' lists of unvisited neighbours, qcap entries each
     int qcap;
     int wc[32];          // per-warp child counts

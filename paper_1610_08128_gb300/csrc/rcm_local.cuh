@@ -30,8 +30,13 @@
 // rows in shared memory too) 0.387 -> 0.129 ms; 10,000 graphs of 100 to 50,000 vertices 25.7 -> 13.7 ms;
 // 500 of them 5.4 -> 2.7 ms; twenty components of 60,000 vertices each 16.3 -> 8.3 ms.
 //
-// Levels with more new vertices than the lists or the table take claim through the graph's global
-// claim words instead (wide_level), level by level, with the same result.
+// At a level with more new vertices than the lists or the table take, a CTA engine's sweep goes on in global
+// memory (run_wide_rest): its vertices are marked there, and the levels that follow are likely as wide. With
+// every such level tried here first and then claimed through the graph's global claim words (wide_level,
+// which looks the rows up three times and reads long ones one after another), 500 random graphs of up to
+// 50,000 vertices and degree 8 took 18.1 ms instead of 6.1, 2,000 power-law ones of up to 20,000 vertices 33
+// instead of 13, a served one of 500,000 vertices 227 instead of 79. The grid's runs end before their levels
+// get that wide, and with direct claims only the lists can be too small: there wide_level takes the level.
 #pragma once
 
 #include "rcm_engine_state.cuh"
@@ -761,13 +766,21 @@ struct Local {
 
     // Labelled levels from level d of F vertices at labels lstart.., held in cache buffer cb, until one is
     // the last (returns true: F and lstart are its) or the next has at least `hi` vertices or is level
-    // `stop` (returns false: they are the next one's). `bad` is set where a label left the graph.
-    __device__ bool labelled_levels(int& F, int& lstart, int& cb, int& d, int hi, int stop, bool& bad) {
+    // `stop` (returns false: they are the next one's). `bad` is set where a label left the graph. Levels too
+    // wide for the lists or the table claim in global memory; with kLeave the first of them ends the loop
+    // instead (`wide`; F and lstart are its, nothing of it done).
+    template <bool kLeave>
+    __device__ bool labelled_levels(int& F, int& lstart, int& cb, int& d, int hi, int stop, bool& bad, bool& wide) {
         const unsigned c0 = s_addr(sm->cache[0]);
         int left = stop - d;  // counted down in place of a level number
         while (true) {
             next_generation();
             int kids = labelled_level(F, lstart, c0 + 4 * kCache * cb, c0 + 4 * kCache * (cb ^ 1), bad);
+            if (kLeave && kids < 0) {
+                wide = true;
+                d = stop - left;
+                return false;
+            }
             if (kids < 0) {
                 __syncthreads();  // every thread has read the counts
                 kids = local_wide_level<kDirect>(a, sm, F, lstart, cb, gen, seq);
@@ -794,18 +807,20 @@ struct Local {
     }
 
     // Labelled sweep from root with labels from nv: eccentricity, last level's min key, size. Returns
-    // false when a label left the graph.
-    __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size) {
+    // false when a label left the graph. rest > 0: it ended before level ecc, of `rest` vertices (the last
+    // of the size numbered), which is too wide (never with direct claims).
+    __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size, int& rest) {
         start(root);
         if (threadIdx.x == 0) perm_end[-nv] = root;
         __syncthreads();
         ++seq;
         int F = 1, cb = 0, lstart = nv;
-        bool bad = false;
+        bool bad = false, wide = false;
         ecc = 0;
-        labelled_levels(F, lstart, cb, ecc, kIntMax, kIntMax, bad);
-        last_key = labelled_key(F, lstart, cb);
+        labelled_levels<!kDirect>(F, lstart, cb, ecc, kIntMax, kIntMax, bad, wide);
+        if (!wide) last_key = labelled_key(F, lstart, cb);
         size = lstart + F - nv;
+        rest = wide ? F : 0;
         return !__syncthreads_or(bad);
     }
 
@@ -838,8 +853,8 @@ struct Local {
         ++seq;
         const int d0 = d;
         int cb = 0;
-        bool bad = false;
-        const bool end = labelled_levels(F, lstart, cb, d, hi, a->probe > d ? a->probe : kIntMax, bad);
+        bool bad = false, wide = false;
+        const bool end = labelled_levels<false>(F, lstart, cb, d, hi, a->probe > d ? a->probe : kIntMax, bad, wide);
         const unsigned long long key = end ? labelled_key(F, lstart, cb) : kKeyMax;
         bad = __syncthreads_or(bad);
         save();
@@ -865,16 +880,17 @@ __device__ __noinline__ int local_wide_level(const EngineArgs* a, EngineSmem* sm
     return l.wide_level(F, lstart, s_addr(sm->cache[cb]), s_addr(sm->cache[cb ^ 1]));
 }
 
-// The sweeps out of line, one register allocation of their own; results in sm->wr. sweep 0: levels-only.
+// The sweeps out of line, one register allocation of their own; results in sm->wr, what a labelled one left
+// in sm->loc.rest. labelled 0: levels-only.
 template <bool kDirect>
 __device__ __noinline__ void local_sweep(const EngineArgs* a, EngineSmem* sm, int labelled, int root, int nv) {
     Local<kDirect> l(a, sm);
-    int ecc = 0, size = 0;
+    int ecc = 0, size = 0, rest = 0;
     unsigned long long key = kKeyMax;
     long long reached = 0;
     bool ok = true;
     if (labelled) {
-        ok = l.sweep_labelled(root, nv, ecc, key, size);
+        ok = l.sweep_labelled(root, nv, ecc, key, size, rest);
         reached = size;
     } else {
         l.sweep_levels(root, ecc, key, reached);
@@ -885,6 +901,7 @@ __device__ __noinline__ void local_sweep(const EngineArgs* a, EngineSmem* sm, in
         sm->wr.lk = key;
         sm->wr.reached = reached;
         sm->wr.bad = ok ? 0 : 1;
+        sm->loc.rest = rest;
     }
     __syncthreads();
 }

@@ -99,7 +99,9 @@ static const void* single_kernel(int threads, bool async = false, bool hybrid = 
 // k_rcm_components: the most hash slots, the list entries of a component's local sweeps and the most dynamic
 // shared memory it may take (with its static part under the 227 KB of a CTA: graphs of up to 1.4M
 // vertices).
-constexpr int kComponentSlots = 8192;
+// (4,096 slots leave L1 to the levels beyond the lists: four 60^3 grids beside each other 16.3 -> 10.3 ms.)
+constexpr int kComponentSlots = 4096;
+constexpr int kGridSlots = 8192;  // the grid kernel's table
 constexpr int kComponentEntries = 3072;
 constexpr size_t kComponentSmem = 206 * 1024;
 // The grid kernel's table leaves every CTA's wide levels some L1 where it can (they read their rows
@@ -531,7 +533,7 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
     args.gvis = (unsigned*)(base + align16(L.pool4 + 12 * (size_t)n));
     size_t dyn = kSingleDynSmem;
     if (sl.local) {
-        int slots = kComponentSlots;
+        int slots = kGridSlots;
         while (slots > 2048 && local_bytes(n, slots, kComponentEntries) > kGridLocalSmem) slots /= 2;
         const size_t bytes = local_bytes(n, slots, kComponentEntries);
         if (bytes <= kComponentSmem) {

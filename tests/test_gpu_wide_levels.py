@@ -1,0 +1,84 @@
+"""CTA engines (batches, served requests, components) on graphs whose levels outgrow the shared lists and
+table: the sweep goes on in global memory from the first such level, through levels that get narrow again,
+and every sweep but the last leaves nothing behind. Orderings equal the serial oracle's, exactly."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1610_08128_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rcm():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1610_08128_gb300 import build, rcm
+
+    build.build()
+    rcm.load()
+    return rcm
+
+
+def device(x):
+    return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+def necklace(bulbs, width, seed):
+    """Wide stars joined by paths: levels of `width` vertices with levels of one between them."""
+    src, dst, at = [], [], 0
+    for _ in range(bulbs):
+        hub, ring, sink = at, np.arange(at + 1, at + 1 + width), at + 1 + width
+        src += [np.full(width, hub), ring, np.array([sink, sink + 1])]
+        dst += [ring, np.full(width, sink), np.array([sink + 1, sink + 2])]
+        at = sink + 2
+    g = synth.csr_from_edges(at + 1, np.concatenate(src), np.concatenate(dst))
+    return synth.permute(g, synth.random_permutation(g.n, seed))
+
+
+def beside(parts, seed):
+    b = synth.concat(parts)
+    return synth.permute(synth.Csr(b.n, b.rowptr, b.colidx), synth.random_permutation(b.n, seed))
+
+
+GRAPHS = {
+    "grid3d_60": lambda: synth.grid((60, 60, 60), seed=1),             # 2,700 vertices in the widest level
+    "grid3d_45": lambda: synth.grid((45, 45, 45), seed=2),             # 1,500: at the lists' edge
+    "degree_8": lambda: synth.random_graph(20_000, 80_000, seed=3, connected=True),
+    "degree_30": lambda: synth.random_graph(6000, 90_000, seed=4, connected=True),
+    "power_law": lambda: synth.power_law(20_000, 10.0, 2.5, 5),        # hubs, and small components
+    "necklace_2047": lambda: necklace(4, 2047, 6),
+    "necklace_2049": lambda: necklace(4, 2049, 7),
+    "necklace_700": lambda: necklace(9, 700, 8),
+    "two_wide_parts": lambda: beside([synth.random_graph(9000, 40_000, seed=9, connected=True),
+                                      synth.grid((50, 50, 50), seed=10), synth.path(700, seed=11)], 12),
+}
+
+
+@pytest.mark.parametrize("threads", [0, 128, 256, 512])
+def test_batch(rcm, threads):
+    graphs = [make() for make in GRAPHS.values()]
+    b = synth.concat(graphs)
+    o = rcm.rcm_batch_options()
+    o.block_threads = threads
+    perm = torch.empty(b.n, dtype=torch.int32, device="cuda")
+    rcm.check(rcm.rcm_order_batch_ex(b.G, b.n, device(b.goff), device(b.rowptr), device(b.colidx), perm, o))
+    rcm.check(rcm.rcm_stream_status())
+    host = perm.cpu().numpy()
+    for i, (name, g) in enumerate(zip(GRAPHS, graphs)):
+        assert np.array_equal(host[b.goff[i]:b.goff[i + 1]], oracle.rcm(g.n, g.rowptr, g.colidx)), name
+
+
+@pytest.mark.parametrize("fused", [0, -1, 2])
+def test_components(rcm, fused):
+    """Wide components beside each other, none of them 3/4 of the vertices."""
+    g = beside([make() for make in GRAPHS.values()], 13)
+    o = rcm.rcm_options()
+    o.fused_sweeps, o.components_first = fused, 1
+    got, stats = rcm.order(device(g.rowptr), device(g.colidx), o, with_stats=True)
+    want, ref = oracle.rcm(g.n, g.rowptr, g.colidx, with_stats=True)
+    assert np.array_equal(got.cpu().numpy(), want)
+    assert stats["components"] == ref["components"]
+    assert stats["sweeps"] == ref["sweeps"] - 2 * ref["isolated"]  # (the oracle counts two for an isolated vertex)
