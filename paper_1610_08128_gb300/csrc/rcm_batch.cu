@@ -23,6 +23,10 @@ namespace rcm {
 constexpr int kBatchEntries = 3072;
 constexpr int kBatchSlots = 4096;
 constexpr int kBatchMinSlots = 2048;
+// What a launch takes of an SM where its largest graph is beyond the largest bitmap (1.46M vertices): that
+// graph takes the longest, all in global memory, and wants L1 (graphs of 1.2M, 1.7M and 2.5M vertices: 165 ms
+// with the largest bitmap, 98 so; 137 on the 256 threads that were the default before the local sweeps).
+constexpr int kBatchLeanSmem = 128 * 1024;
 constexpr int kBatchStaticSmem = 18 * 1024;  // EngineSmem and the rest, rounded up
 constexpr int kSmemPerSm = 227 * 1024;
 
@@ -33,10 +37,13 @@ struct LocalShape {
 };
 static LocalShape local_shape(int max_n, int G, int per_sm, int sms) {
     const int want = std::max(1, std::min(per_sm, (G + sms - 1) / sms));
-    const long long bytes = kSmemPerSm / want - 1024 - kBatchStaticSmem;
-    const long long bitmap = bytes - (long long)local_bytes(0, kBatchMinSlots, kBatchEntries);
-    LocalShape l{(int)std::min<long long>(std::min(max_n, kLocalMax), std::max<long long>(0, bitmap / 16 * 128)),
-                 kBatchMinSlots};
+    auto shape = [&](long long bytes) {
+        const long long bitmap = bytes - (long long)local_bytes(0, kBatchMinSlots, kBatchEntries);
+        return (int)std::min<long long>(std::min(max_n, kLocalMax), std::max<long long>(0, bitmap / 16 * 128));
+    };
+    long long bytes = kSmemPerSm / want - 1024 - kBatchStaticSmem;
+    if (want == 1 && shape(bytes) < max_n) bytes = kBatchLeanSmem - 1024 - kBatchStaticSmem;
+    LocalShape l{shape(bytes), kBatchMinSlots};
     while (l.slots < kBatchSlots && (long long)local_bytes(l.cap, 2 * l.slots, kBatchEntries) <= bytes) l.slots *= 2;
     return l;
 }

@@ -82,3 +82,64 @@ def test_components(rcm, fused):
     assert np.array_equal(got.cpu().numpy(), want)
     assert stats["components"] == ref["components"]
     assert stats["sweeps"] == ref["sweeps"] - 2 * ref["isolated"]  # (the oracle counts two for an isolated vertex)
+
+
+# What a bitmap takes at most: 1.46M vertices with one CTA on an SM, 0.54M with two (256 threads), 0.08M with
+# four (128 threads); a launch whose largest graph is beyond it sizes the others' state smaller.
+BEYOND = {
+    "one_per_sm": (512, [(1300, 1250), (900, 800), (120, 130)], 0),
+    "from_the_sizes": (0, [(1300, 1250), (900, 800), (120, 130)], 0),
+    "one_per_sm_256": (256, [(1300, 1250), (900, 800), (120, 130)], 0),
+    "two_per_sm": (256, [(800, 700), (700, 690), (60, 70)], 350),
+    "four_per_sm": (128, [(300, 280), (280, 270), (60, 70)], 700),
+}
+
+
+@pytest.mark.parametrize("name", list(BEYOND))
+def test_graphs_beyond_the_bitmap(rcm, name):
+    threads, grids, small = BEYOND[name]
+    graphs = [synth.grid_fast(d, seed=i) for i, d in enumerate(grids)] + [synth.path(3, seed=i) for i in range(small)]
+    b = synth.concat(graphs)
+    o = rcm.rcm_batch_options()
+    o.block_threads = threads
+    perm = torch.empty(b.n, dtype=torch.int32, device="cuda")
+    rcm.check(rcm.rcm_order_batch_ex(b.G, b.n, device(b.goff), device(b.rowptr), device(b.colidx), perm, o))
+    rcm.check(rcm.rcm_stream_status())
+    host = perm.cpu().numpy()
+    for i, g in enumerate(graphs):
+        assert np.array_equal(host[b.goff[i]:b.goff[i + 1]], oracle.rcm(g.n, g.rowptr, g.colidx)), i
+
+
+def with_diagonal(g, rows):
+    """The pattern with its first `rows` rows' diagonals stored too."""
+    at = np.arange(rows)
+    colidx = np.insert(g.colidx, g.rowptr[:rows], at).astype(np.int32)
+    return g.rowptr + np.minimum(np.arange(g.n + 1), rows).astype(np.int32), colidx
+
+
+def test_plan_whose_graphs_grow_beyond_its_bitmap(rcm):
+    """A plan made for graphs of 300 vertices, replayed after its buffers were filled with a pattern of the
+    same size that has one graph of 20,000 vertices."""
+    even = synth.concat([synth.grid((15, 20), seed=i) for i in range(80)])
+    grown = synth.concat([synth.grid((100, 200), seed=99)] + [synth.path(50, seed=i) for i in range(80)])
+    assert even.n == grown.n and len(grown.colidx) < len(even.colidx)
+    rowptr, colidx = with_diagonal(grown, len(even.colidx) - len(grown.colidx))
+    fills = [(np.append(even.goff, even.n), even.rowptr, even.colidx), (grown.goff, rowptr, colidx)]
+    goff, rp, ci = (device(x) for x in fills[0])
+    perm = torch.empty(even.n, dtype=torch.int32, device="cuda")
+    st, plan = rcm.rcm_batch_plan_create(len(goff) - 1, even.n, len(ci), goff, rp, ci, perm)
+    rcm.check(st, "plan")
+    try:
+        for at in (0, 1, 0):
+            for buf, x in zip((goff, rp, ci), fills[at]):
+                buf.copy_(torch.from_numpy(np.ascontiguousarray(x)))
+            rcm.check(rcm.rcm_batch_plan_launch(plan))
+            rcm.check(rcm.rcm_batch_plan_status(plan))
+            host = perm.cpu().numpy()
+            for lo, hi in zip(fills[at][0][:-1], fills[at][0][1:]):
+                if hi == lo:
+                    continue
+                r = fills[at][1][lo:hi + 1]
+                assert np.array_equal(host[lo:hi], oracle.rcm(int(hi - lo), r - r[0], fills[at][2][r[0]:r[-1]] - lo))
+    finally:
+        rcm.check(rcm.rcm_batch_plan_destroy(plan))
