@@ -13,10 +13,12 @@ constexpr int kWarpLevel = 32;  // narrow levels of at most this many vertices r
 // A level of a few hundred vertices that holds a hub is far more work than one CTA does quickly,
 // and a labelled first sweep over hubs costs more than a levels-only one: graphs with a vertex of
 // more than kHubDegree neighbours take a lower frontier switch and levels-only first sweeps by
-// default, and their whole-grid levels spread long rows over a CTA's warps (Engine::hub_round: a
-// 1M-vertex power-law graph with hubs of 7,000 entries 11.3 -> 6.2 ms a call; 24 ms with the grid's
-// defaults).
+// default (24 -> 11.3 ms a call on a 1M-vertex power-law graph with hubs of 7,000 entries). Where their rows
+// hold one entry in kHubShare or more, the whole-grid levels also spread long rows over a CTA's warps
+// (Engine::hub_round: 6.7 ms); a few dense rows in a grid do not pay for its barriers in every round (a 192^3
+// grid with one row of 600 entries 5.02 ms without, 5.66 with).
 constexpr int kHubDegree = 512;
+constexpr int kHubShare = 1024;
 // Patterns this sparse may fall into parts: 2-nearest-neighbour meshes and their spanning trees have
 // 2.7 neighbours a row, 3-nearest ones 3.7, grids 4 and 6. The probe sweep from the first start vertex runs
 // one part while everything else waits (1.2M-point mesh in 20 strips 9.6 ms with it, 8.0 without); the
@@ -56,8 +58,8 @@ struct EngineArgs {
     int fused;
     int cc_first;                // persistent grid: build the component table before the first sweep (-1: where
                                  // the rows average fewer than kPartsDegree / 10 neighbours and the probe gives up)
-    int hubs;                    // whole grid: the graph has a vertex of more than kHubDegree neighbours (set on
-                                 // the device)
+    int hubs;                    // whole grid: rows of more than kHubDegree neighbours hold one entry in kHubShare
+                                 // or more (set on the device)
     int hub_auto;                // default launch of the persistent grid: a graph with a vertex of more
                                  // than kHubDegree neighbours takes the frontier switch kHubNarrow and
                                  // levels-only first sweeps (decided on the device from ctl->maxdeg)

@@ -68,6 +68,7 @@ struct alignas(128) Ctl {
     long long phase_ns[8];         // per-phase time of CTA 0 (profile_phases)
     ExSlot slots[2][kMaxGridBlocks];  // exchange slots, double-buffered by epoch parity
     int counts[2][kMaxGridBlocks];    // the counts-only exchange's
+    unsigned long long hubsum;        // off-diagonal entries of rows with more than kHubDegree
 };
 
 // Counters of the asynchronous levels-only sweep (one per ordering), each hot word on its own

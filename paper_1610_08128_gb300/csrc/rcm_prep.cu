@@ -10,6 +10,7 @@
 //    owns come out already in (degree, id) order, so the new level is ordered by (parent label,
 //    degree, id) by a prefix sum over parents alone.
 //  * k_bw_scatter / k_bw_rows: bandwidth and profile of P A P^T (Sec. II-A).
+#include "rcm_engine_state.cuh"
 #include "rcm_prep.cuh"
 
 namespace rcm {
@@ -116,6 +117,7 @@ __global__ void k_degree_validate(int n, int nnz, const int* __restrict__ rowptr
         if (adist) adist[v] = ~0ull;
         if (fkey) fkey[v] = 0;
         local_max = max(local_max, d);
+        if (d > kHubDegree) atomicAdd(&ctl->hubsum, (unsigned long long)d);
         local_sum += (unsigned)d;
     }
     __syncwarp();

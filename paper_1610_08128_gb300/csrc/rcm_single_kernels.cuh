@@ -76,7 +76,7 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
         if (threadIdx.x == 0) {
             // a level with a hub fits neither the local lists nor the table, and a graph with hubs has few
             // levels for them to speed up (1M-vertex power-law graph: 13.8 ms without, 19.5 with)
-            smem.args.hubs = 1;
+            smem.args.hubs = ctl->hubsum * kHubShare >= ctl->degsum ? 1 : 0;
             smem.hub = (int*)s_sort;  // idle during a sweep
             smem.args.local_hi = 0;
             if (args.hub_auto) {

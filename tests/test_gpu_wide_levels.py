@@ -143,3 +143,22 @@ def test_plan_whose_graphs_grow_beyond_its_bitmap(rcm):
                 assert np.array_equal(host[lo:hi], oracle.rcm(int(hi - lo), r - r[0], fills[at][2][r[0]:r[-1]] - lo))
     finally:
         rcm.check(rcm.rcm_batch_plan_destroy(plan))
+
+
+@pytest.mark.parametrize("rows,length", [(1, 513), (1, 600), (1, 5000), (2, 1000), (12, 520), (40, 900)])
+def test_grid_with_dense_rows(rcm, rows, length):
+    """Rows of more than 512 entries in a grid, from one in ten thousand entries to one in ten: on both sides
+    of the share from which the grid kernel spreads long rows over its warps."""
+    g = synth.grid((70, 70, 70))
+    rng = synth.rng_for([21, rows, length])
+    src = np.repeat(np.arange(g.n), np.diff(g.rowptr))
+    hubs = rng.choice(g.n, rows, replace=False)
+    ends = np.concatenate([rng.choice(g.n, length, replace=False) for _ in range(rows)])
+    h = synth.csr_from_edges(g.n, np.concatenate([src, np.repeat(hubs, length)]), np.concatenate([g.colidx, ends]))
+    h = synth.permute(h, synth.random_permutation(h.n, [22, rows]))
+    want = oracle.rcm(h.n, h.rowptr, h.colidx)
+    for narrow in (0, -1, 700):
+        o = rcm.rcm_options()
+        o.narrow_threshold = narrow
+        got = rcm.order(device(h.rowptr), device(h.colidx), o).cpu().numpy()
+        assert np.array_equal(got, want), narrow
