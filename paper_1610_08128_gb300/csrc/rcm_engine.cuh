@@ -418,8 +418,11 @@ struct Engine {
             int x = 0, y = 0, mx = 0;
             unsigned long long k = kKeyMax;
             if (payload && !bad) {
-                // slots in batches of 8 per lane: all loads of a batch are issued before use
-                for (int i0 = threadIdx.x; i0 < B; i0 += 32 * 8) {
+                // slots in batches of 8 per lane: all loads of a batch are issued before use (every lane
+                // takes every batch: where those beyond the last slot skipped it, on fewer than 32 CTAs,
+                // the warp's reduction below took 3 us longer)
+                for (int base = 0; base < B; base += 32 * 8) {
+                    const int i0 = base + (int)threadIdx.x;
                     unsigned long long f[8], kk[8];
 #pragma unroll
                     for (int t = 0; t < 8; ++t) {
@@ -504,7 +507,8 @@ struct Engine {
             }
             __syncwarp();
             int x = 0, y = 0, mx = 0;
-            for (int i0 = threadIdx.x; i0 < B; i0 += 32 * 8) {
+            for (int base = 0; base < B; base += 32 * 8) {
+                const int i0 = base + (int)threadIdx.x;
                 int v[8];
 #pragma unroll
                 for (int t = 0; t < 8; ++t) v[t] = i0 + 32 * t < B ? ldcg(at + i0 + 32 * t) : 0;
