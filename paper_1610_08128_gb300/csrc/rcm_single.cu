@@ -107,6 +107,9 @@ constexpr size_t kComponentSmem = 206 * 1024;
 // The grid kernel's table leaves every CTA's wide levels some L1 where it can (they read their rows
 // twice): a 1M-vertex power-law graph 3.99 ms with 96 KB of shared memory, 4.24 with 201.
 constexpr size_t kGridLocalSmem = 170 * 1024;
+// A cluster's few CTAs run wide levels for long: a 100^3 grid on 16 CTAs 3.6 ms with no more than this (the
+// local state then stays off), 4.5 with 206 KB; a 750^2 grid 9.4 with the state and a small table, 10.5 without.
+constexpr size_t kClusterSmem = 128 * 1024;
 constexpr size_t kComponentSmem2 = 94 * 1024;  // the most with two CTAs on an SM
 
 constexpr int kSingleDynSmem = (int)((sizeof(unsigned long long) + sizeof(int)) * kCompSmem);
@@ -147,7 +150,7 @@ int single_cluster_max() {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(c);
             cfg.blockDim = dim3(512);
-            cfg.dynamicSmemBytes = kSingleDynSmem;
+            cfg.dynamicSmemBytes = kClusterSmem;  // the most a launch takes (enqueue_single)
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = c;
@@ -533,10 +536,11 @@ cudaError_t enqueue_single(int n, long long nnz, const int* rowptr, const int* c
     args.gvis = (unsigned*)(base + align16(L.pool4 + 12 * (size_t)n));
     size_t dyn = kSingleDynSmem;
     if (sl.local) {
+        const size_t good = sl.cluster ? kSingleDynSmem : kGridLocalSmem, most = sl.cluster ? kClusterSmem : kComponentSmem;
         int slots = kGridSlots;
-        while (slots > 2048 && local_bytes(n, slots, kComponentEntries) > kGridLocalSmem) slots /= 2;
+        while (slots > 2048 && local_bytes(n, slots, kComponentEntries) > good) slots /= 2;
         const size_t bytes = local_bytes(n, slots, kComponentEntries);
-        if (bytes <= kComponentSmem) {
+        if (bytes <= most) {
             args.local_hi = std::min(sl.narrow + sl.narrow / 2, kCache);
             args.local_slots = slots;
             args.local_entries = kComponentEntries;

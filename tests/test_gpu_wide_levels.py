@@ -162,3 +162,14 @@ def test_grid_with_dense_rows(rcm, rows, length):
         o.narrow_threshold = narrow
         got = rcm.order(device(h.rowptr), device(h.colidx), o).cpu().numpy()
         assert np.array_equal(got, want), narrow
+
+
+@pytest.mark.parametrize("blocks", [2, 8, 0])
+@pytest.mark.parametrize("side", [100, 880, 960])
+def test_cluster_beside_its_shared_memory(rcm, side, blocks):
+    """One cluster on graphs whose bitmap fits beside the full table, beside a small one, and not at all."""
+    g = synth.grid_fast((side, side), seed=side)
+    o = rcm.rcm_options()
+    o.executor, o.cluster, o.grid_blocks = 1, 1, blocks
+    got = rcm.order(device(g.rowptr), device(g.colidx), o).cpu().numpy()
+    assert np.array_equal(got, oracle.rcm(g.n, g.rowptr, g.colidx))
