@@ -1201,11 +1201,10 @@ struct Engine {
     }
 
     // Levels-only sweep from root. On return: ecc, the min (degree, id) key of the last level and
-    // the number of vertices reached (the component's size). With a->probe set (whole grid) the sweep gives
-    // up with ecc = -1 where that level is still narrow (see component).
+    // the number of vertices reached (the component's size).
     __device__ bool sweep_levels(int root, int& ecc, unsigned long long& last_key, long long& reached) {
         if constexpr (kAsync) {
-            if (a->adist && async_ok && a->probe == 0) {
+            if (a->adist && async_ok) {
                 const int rc = sweep_async(root, ecc, last_key, reached);
                 if (rc >= 0) return rc == 1;
                 async_ok = false;  // the queue ran full: this and later sweeps run level by level
@@ -1236,7 +1235,6 @@ struct Engine {
             if (kCtaOnly || F < a->narrow_thr) {
                 unsigned long long lk = kKeyMax;
                 if (kCtaOnly || b == 0) {
-                    const int stop = !kCtaOnly && a->probe > ecc ? a->probe : kIntMax;
                     if (!in_cache) {
                         for (int i = threadIdx.x; i < F; i += blockDim.x) sm->cache[cb][i] = ldcg(cur + i);
                         in_cache = true;
@@ -1290,7 +1288,7 @@ struct Engine {
                             fail_at(kSiteLevels, ecc);
                             return false;
                         }
-                        if (!kCtaOnly && (F >= a->narrow_thr || ecc >= stop)) break;
+                        if (!kCtaOnly && F >= a->narrow_thr) break;
                     }
                     if (kCtaOnly) {
                         __syncthreads();
@@ -1299,7 +1297,7 @@ struct Engine {
                     }
                     if (threadIdx.x == 0) {
                         c->pub_F = F;
-                        c->pub_cur = (cur == a->qb ? 1 : 0) | (F > 0 && ecc >= stop ? 2 : 0);
+                        c->pub_cur = (cur == a->qb) ? 1 : 0;
                         c->pub_ecc = ecc;
                         c->pub_key = lk;
                         c->pub_reached = reached;
@@ -1321,15 +1319,11 @@ struct Engine {
                 lk = sm->bck;
                 reached = __ldcg(&c->pub_reached);
                 __syncthreads();
-                cur = (pc & 1) ? a->qb : a->qa;
-                nxt = (pc & 1) ? a->qa : a->qb;
+                cur = pc ? a->qb : a->qa;
+                nxt = pc ? a->qa : a->qb;
                 in_cache = false;
                 if (Fp == 0) {
                     last_key = lk;
-                    return true;
-                }
-                if (pc & 2) {
-                    ecc = -1;
                     return true;
                 }
                 F = Fp;
@@ -1839,7 +1833,8 @@ struct Engine {
 
     // Labelled sweep from root, labels from nv. On return: ecc, the min (degree, id) key of the
     // last level, and the component size (labels nv .. nv+size-1). With a->probe set (whole grid) the sweep
-    // gives up with ecc = -1 and size the vertices numbered so far where that level is still narrow.
+    // gives up with ecc = -1 and size the vertices numbered so far where that level is still narrow and they
+    // are less than 3/4 of the vertices left.
     // F0 > 0 (CTA engines): the sweep goes on at level d0, F0 vertices at labels from lstart0, with the
     // vertices numbered so far marked.
     __device__ bool sweep_labelled(int root, int nv, int& ecc, unsigned long long& last_key, int& size, int d0 = 0,
@@ -1962,7 +1957,7 @@ struct Engine {
                         c->pub_start = lstart;
                         c->pub_ecc = d;
                         c->pub_key = lk;
-                        c->pub_lastF = F > 0 && d >= stop ? -1 : lastF;
+                        c->pub_lastF = F > 0 && d >= stop && 4LL * (lstart + F - nv) < 3LL * (a->n - nv) ? -1 : lastF;
                         c->pub_reached = from;
                         c->qtail[0] = c->qtail[1] = c->qtail[2] = 0;
                     }
@@ -2326,8 +2321,7 @@ struct Engine {
     // all_left >= 0 (the number of vertices not yet numbered), the call stops after the first
     // sweep when the component is smaller than that, is small enough for the component table to
     // order it at least as fast, and holds less than 3/4 of the vertices left, returning
-    // size = -1 (nothing numbered). With a->probe set it also stops where that level of the sweep is still
-    // narrow (on the whole grid): size = minus the vertices reached by then.
+    // size = -1 (nothing numbered), also where a first sweep that is a probe gave up.
     __device__ bool component(int r, int nv, int& size, long long all_left = -1) {
         if (!in_graph(r) || nv < 0 || nv >= a->n) {
             fail_at(kSiteStart, r);
@@ -2348,14 +2342,6 @@ struct Engine {
             tick(kPhOther);
         } else if (!levels(r, ecc_prev, k1, reached)) {
             return false;
-        }
-        if constexpr (!kCtaOnly) {
-            if (threadIdx.x == 0) sm->args.probe = 0;  // (every sweep ends with a barrier)
-            __syncthreads();
-            if (ecc_prev < 0) {  // gave up
-                size = -(int)reached;
-                return true;
-            }
         }
         // The start vertex's component does not hold every vertex left: the others get a component
         // table. The component is finished here, its sweep kept, when the table would order it no
@@ -2944,6 +2930,7 @@ __device__ __noinline__ bool run_grid_labelled(const EngineArgs* a, EngineSmem* 
     if (!e.sweep_labelled(root, nv, ecc, key, size)) return false;
     __syncthreads();
     if (threadIdx.x == 0) {
+        sm->args.probe = 0;  // the first sweep only
         sm->sw.ecc = ecc;
         sm->sw.key = key;
         sm->sw.size = size;

@@ -65,6 +65,8 @@ struct EngineArgs {
                                  // levels-only first sweeps (decided on the device from ctl->maxdeg)
     int obits;                   // low bits of a key holding the in-level order
     int profile;                 // accumulate per-phase time (CTA 0, thread 0)
+    int probe;                   // whole grid: a level at which a sweep that is still narrow gives up (0 = none; set
+                                 // on the device)
     long long limit_ns;
     // concurrent components (whole-grid executor only)
     int* cc_parent;              // n ints
@@ -95,8 +97,6 @@ struct EngineArgs {
     int local_hi;                // a run ends at a level of this many vertices (narrow_thr starts one)
     int local_slots, local_entries;
     unsigned* gvis;              // bitmap of n vertices: what the grid's levels visited, for the next run
-    int probe;                   // whole grid: a level at which a sweep that is still narrow gives up (0 = none; set
-                                 // on the device)
 };
 
 enum { kPhExpand = 0, kPhClaim, kPhOwn, kPhLabels, kPhExchange, kPhRedist, kPhWaitNarrow, kPhOther };
@@ -111,10 +111,10 @@ struct LocalState {
     unsigned* hval;      // ((gmax - generation) << idbits) | smallest frontier position
     unsigned gen;        // generation of the last labelled level
     unsigned seq;        // labelled sweeps so far (tags the global claims)
-    int rest;            // vertices of the level at which the last sweep went on in global memory (0 = it did not)
     unsigned* list;      // the warps' lists of unvisited neighbours, qcap entries each
     int qcap;
     int wc[32];          // per-warp child counts
+    int rest;            // vertices of the level at which the last sweep went on in global memory (0 = it did not)
 };
 
 // Shared memory of one engine CTA.

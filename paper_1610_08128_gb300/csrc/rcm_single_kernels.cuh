@@ -96,8 +96,15 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
     // the pattern only looks like several parts, a probe decides, which gives up while it is cheap
     const bool sparse = __ldcg(&ctl->degsum) * 10 < (unsigned long long)n * kPartsDegree;
     bool first = args.cc_first <= 0, tried = false, thin = false;
+    const int fused = smem.args.fused;
+    __syncthreads();
     if (args.cc_first < 0 && sparse && args.cc_cap > 0) {
-        if (threadIdx.x == 0) smem.args.probe = kProbeLevels;
+        // (the probe is a labelled sweep; without fused sweeps: the table first)
+        if (fused == 0) first = false;
+        else if (threadIdx.x == 0) {
+            smem.args.probe = kProbeLevels;
+            smem.args.fused = 2;
+        }
         __syncthreads();
     }
     while (nv < n) {
@@ -126,8 +133,9 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
         const long long left = (first && args.cc_cap > 0) ? (long long)(n - nv) : -1;
         first = false;
         if (!e.component((int)(unsigned)(k0 & 0xffffffffu), nv, size, left)) return;
+        if (threadIdx.x == 0) smem.args.fused = fused;
         if (size < 0) {  // more components, or a long one: the next iteration prepares them all
-            thin = size < -1 && -size <= kProbeLevels * kThinLevel;
+            thin = smem.sw.ecc < 0 && smem.sw.size <= kProbeLevels * kThinLevel;
             continue;
         }
         // runs of local levels leave no claims: the vertices just numbered are marked for the searches
