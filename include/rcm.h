@@ -338,7 +338,8 @@ rcm_status rcm_server_create(size_t hbm_budget_bytes, int32_t max_inflight, rcm_
 typedef struct {
     int64_t cluster_min_vertices; /* requests of at least this many vertices run the persistent
                                      engine of rcm_order launched as one thread-block cluster;
-                                     smaller ones run on one CTA. 0 = 1,048,576; -1 = never       */
+                                     smaller ones run on one CTA. 0 = 1,048,576, or 524,288 while
+                                     at most 8 requests are in the server; -1 = never             */
     int32_t cluster_blocks;       /* CTAs of that cluster, 2..16 as the device allows; 0 = 4, or 8
                                      while at most 64 requests are in the server                  */
     int32_t debug_fail_after;     /* test hook: once this many requests have completed, the server

@@ -7,8 +7,8 @@
 //    caller's buffer is in host memory), a status word and the workspace of the ordering.
 //    Requests are admitted in arrival order whenever a region and an in-flight slot are free; a
 //    request larger than the whole budget is refused at submission (RCM_ERR_TOO_LARGE).
-//  * Execution: each admitted request gets its own stream. Requests below kServeClusterMin
-//    vertices run as a batch of one graph: the validation and sorted-row kernels, then the batched
+//  * Execution: each admitted request gets its own stream. All but the largest (rcm_serve_policy.hpp)
+//    run as a batch of one graph: the validation and sorted-row kernels, then the batched
 //    executor with one CTA (Engine<true>, rcm_batch.cu). Larger ones run the persistent engine of
 //    rcm_order (Engine<false>) launched as one thread-block cluster, whose CTAs the hardware
 //    schedules together, so wide levels spread over several SMs. Requests that arrive while
@@ -34,20 +34,10 @@
 #include "rcm_batch.cuh"
 #include "rcm_host.hpp"
 #include "rcm_internal.cuh"
+#include "rcm_serve_policy.hpp"
 #include "rcm_single.cuh"
 
 namespace rcm {
-
-// Requests of at least kServeClusterMin vertices run on a cluster by default, smaller ones on one CTA. With
-// the one CTA's state in shared memory it orders up to a million vertices in half the SM time a cluster
-// needs. The cluster has kServeClusterBlocks CTAs under load and kServeClusterIdle while at most
-// kServeFew requests are in the server (they would leave SMs idle). GB300, 48 requests of 1,000 to 4M
-// vertices at once: 102 ms with clusters of 4 from 524,288 vertices, 90 from 1,048,576, 75 with 8 CTAs
-// there; 800 requests at once (32 hardware queues, 256 in flight): 1,680, 2,702 and 1,838 orderings/s.
-constexpr int kServeClusterIdle = 8;
-constexpr int kServeFew = 64;
-constexpr long long kServeClusterMin = 1LL << 20;
-constexpr int kServeClusterBlocks = 4;
 
 // Arena bytes of one request: the staged CSR and result when they are in host memory, a 256-byte
 // header holding the graph offsets {0, n} of a batch of one, and the larger of the two executors'
@@ -132,7 +122,7 @@ struct Request {
     size_t off = 0, bytes = 0;
     int slot = -1;
     int state = 0;  // 0 waiting, 1 running, 2 done
-    bool few = false;     // admitted while the server held few requests
+    int load = 0;         // requests in the server when it was admitted
     bool orphan = false;  // finished by the failure path: its host function may still be pending
     rcm_status status = RCM_OK;
     double t_submit = 0, t_start = 0, t_done = 0;
@@ -167,7 +157,7 @@ struct Server {
     long long submitted = 0, completed = 0, failed = 0, cancelled = 0;
     int running = 0, max_running = 0;
     cudaError_t broken = cudaSuccess;  // first stream error seen: the context is unusable
-    long long cluster_min = kServeClusterMin;  // -1: never
+    long long cluster_min = 0;                 // 0: by load, -1: never
     int cluster_blocks = 0;                    // 0: by load
     int debug_fail_after = 0;                  // test hook (rcm_server_options)
     bool trace = false;                // RCM_TRACE_ERRORS set: failed requests are reported on stderr
@@ -261,12 +251,13 @@ static rcm_status launch_request(Server* s, Request* r) {
     SlotHost* hs = &s->h_slots[r->slot];
     hs->status = 0;
     const int* status_dev = nullptr;
-    if (s->cluster_min >= 0 && r->n >= s->cluster_min && single_cluster_max() > 0) {
+    const int cluster = s->cluster_min < 0 ? 0
+                        : serve_cluster(r->n, r->load, s->cluster_min, s->cluster_blocks, single_cluster_max());
+    if (cluster > 0) {
         const SingleLayout L = single_layout(r->n, r->nnz);
         rcm_options o{};
         o.cluster = 1;
-        o.grid_blocks = s->cluster_blocks ? s->cluster_blocks
-                        : r->few ? std::min(kServeClusterIdle, single_cluster_max()) : kServeClusterBlocks;
+        o.grid_blocks = cluster;
         SingleLaunch sl;
         const rcm_status ls = single_launch(r->n, r->nnz, o, &sl);
         if (ls != RCM_OK) return ls;
@@ -277,7 +268,8 @@ static rcm_status launch_request(Server* s, Request* r) {
         hs->goff[0] = 0;
         hs->goff[1] = r->n;
         if (e == cudaSuccess) e = cudaMemcpyAsync(d_goff, hs->goff, sizeof(hs->goff), cudaMemcpyHostToDevice, st);
-        const BatchTuning t;
+        BatchTuning t;
+        t.threads = kServeThreads;
         if (!batch_prepare(t)) return RCM_ERR_CUDA;
         if (e == cudaSuccess) e = enqueue_batch(1, r->n, (int)r->nnz, d_goff, nullptr, rowptr, colidx, perm, ws, L, t, st,
                                                 r->n);
@@ -359,7 +351,7 @@ static void worker_loop(Server* s) {
             r->t_start = now_s();
             s->running++;
             s->max_running = std::max(s->max_running, s->running);
-            r->few = s->running + (int)s->waiting.size() <= kServeFew;
+            r->load = s->running + (int)s->waiting.size();
             admit.push_back(r);
         }
         if (!admit.empty()) {
@@ -446,7 +438,7 @@ rcm_status rcm_server_create_ex(size_t hbm_budget_bytes, int32_t max_inflight, c
     s.alloc.reset(s.budget);
     s.max_inflight = max_inflight;
     if (opts) {
-        s.cluster_min = opts->cluster_min_vertices == 0 ? kServeClusterMin : opts->cluster_min_vertices;
+        s.cluster_min = opts->cluster_min_vertices;
         s.cluster_blocks = opts->cluster_blocks;
         s.debug_fail_after = opts->debug_fail_after;
     }
