@@ -2930,7 +2930,10 @@ __device__ __noinline__ bool run_grid_labelled(const EngineArgs* a, EngineSmem* 
     if (!e.sweep_labelled(root, nv, ecc, key, size)) return false;
     __syncthreads();
     if (threadIdx.x == 0) {
-        sm->args.probe = 0;  // the first sweep only
+        if (sm->args.probe) {  // the first sweep only
+            sm->args.probe = 0;
+            sm->args.fused = sm->sw.fused;
+        }
         sm->sw.ecc = ecc;
         sm->sw.key = key;
         sm->sw.size = size;

@@ -142,6 +142,7 @@ struct EngineSmem {
         unsigned epoch, cepoch;
         int sweep_id, scan_par, ecc, size, prev_start;
         bool async_ok;
+        unsigned char fused;     // args.fused after a probe
         unsigned long long key;
         long long reached;
     } sw;

@@ -96,14 +96,11 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
     // the pattern only looks like several parts, a probe decides, which gives up while it is cheap
     const bool sparse = __ldcg(&ctl->degsum) * 10 < (unsigned long long)n * kPartsDegree;
     bool first = args.cc_first <= 0, tried = false, thin = false;
-    const int fused = smem.args.fused;
-    __syncthreads();
     if (args.cc_first < 0 && sparse && args.cc_cap > 0) {
-        // (the probe is a labelled sweep; without fused sweeps: the table first)
-        if (fused == 0) first = false;
-        else if (threadIdx.x == 0) {
+        if (threadIdx.x == 0) {
+            smem.sw.fused = (unsigned char)smem.args.fused;
             smem.args.probe = kProbeLevels;
-            smem.args.fused = 2;
+            smem.args.fused = 2;  // the probe is a labelled sweep
         }
         __syncthreads();
     }
@@ -133,7 +130,6 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
         const long long left = (first && args.cc_cap > 0) ? (long long)(n - nv) : -1;
         first = false;
         if (!e.component((int)(unsigned)(k0 & 0xffffffffu), nv, size, left)) return;
-        if (threadIdx.x == 0) smem.args.fused = fused;
         if (size < 0) {  // more components, or a long one: the next iteration prepares them all
             thin = smem.sw.ecc < 0 && smem.sw.size <= kProbeLevels * kThinLevel;
             continue;
