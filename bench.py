@@ -98,8 +98,8 @@ def load_peaks():
 
 # the sources of the 512-thread traversal kernel's device code (k_rcm_single); its launch options are
 # recorded beside the traffic figure
-TRAVERSAL_SOURCES = ["rcm_kern_grid512.cu", "rcm_single_kernels.cuh", "rcm_engine.cuh", "rcm_internal.cuh",
-                     "rcm_cc.cuh"]
+TRAVERSAL_SOURCES = ["rcm_kern_grid512.cu", "rcm_single_kernels.cuh", "rcm_engine.cuh", "rcm_engine_state.cuh",
+                     "rcm_local.cuh", "rcm_internal.cuh", "rcm_cc.cuh"]
 
 
 def kernel_sources_hash() -> str:

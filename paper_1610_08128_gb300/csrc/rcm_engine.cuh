@@ -61,11 +61,11 @@ __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// kWarp (CTA engines only; on by default with kSmem): narrow levels of at most kWarpLevel vertices
-// run on warp 0 alone. Off in the engines it slowed through register allocation.
+// kWarp (CTA engines with global state only): narrow levels of at most kWarpLevel vertices run on warp 0
+// alone. Off in the engines it slowed through register allocation.
 // kSmem (CTA engines only): the claims, visit stamps and padded rows of the graph live in shared
-// memory, indexed from the graph's first vertex v0; otherwise they are global arrays indexed by
-// vertex id.
+// memory, indexed from the graph's first vertex v0, and every sweep is a local one (rcm_local.cuh);
+// otherwise they are global arrays indexed by vertex id.
 // kAsync (whole-grid engine only): levels-only sweeps through the asynchronous work queue when
 // the arguments provide it. kBottomUp (whole-grid engine only): each whole-grid level may run
 // bottom-up, chosen per level. Separate instantiations, so the plain top-down kernels carry none
@@ -83,8 +83,8 @@ __device__ __noinline__ void run_warp_labelled(const EngineArgs* a, EngineSmem* 
                                                const int* sh, const int* g, int step);
 
 // Phases A and B for the entries beyond the padded rows of a warp's vertices (u < 0: none on this lane),
-// out of line: most graphs have none, and inlined they cost every level registers (192^3 grid 7.05 against
-// 6.6 ms). Claims; the number of children owned there; those written from position pos on.
+// out of line: most graphs have none, and inlined they cost every level registers (0.4 of the 192^3 grid's
+// 7.0 ms). Claims; the number of children owned there; those written from position pos on.
 template <class Eng>
 __device__ __noinline__ void long_claims(const EngineArgs* a, int u, int dg, unsigned long long key);
 template <class Eng>
@@ -94,7 +94,7 @@ __device__ __noinline__ void long_children(const EngineArgs* a, int u, int dg, u
                                            int lab_base);
 
 // The whole grid's sweeps and, inside the labelled one, its runs of whole-grid levels, out of line: one
-// copy each, with registers of its own (inlined into one kernel they spill: 192^3 grid 7.1 against 6.8
+// copy each, with registers of its own (inlined into one kernel they spill: 0.3 of the 192^3 grid's 7.1
 // ms). Results in sm->sw and sm->wr.
 template <bool kAsync, bool kBottomUp>
 __device__ __noinline__ bool run_grid_levels_only(const EngineArgs* a, EngineSmem* sm, int root);
@@ -110,10 +110,10 @@ __device__ __noinline__ bool run_grid_levels(const EngineArgs* a, EngineSmem* sm
 template <bool kWarp>
 __device__ __noinline__ bool run_wide_rest(const EngineArgs* a, EngineSmem* sm, int root, int nv, int d, int lstart, int F);
 
-template <bool kCtaOnly, bool kSmem = false, bool kAsync = false, bool kBottomUp = false, bool kWarp = kSmem>
+template <bool kCtaOnly, bool kSmem = false, bool kAsync = false, bool kBottomUp = false, bool kWarp = false>
 struct Engine {
     static_assert(kCtaOnly || !kSmem, "shared-memory state needs a CTA engine");
-    static_assert(kCtaOnly || !kWarp, "warp-0 levels need a CTA engine");
+    static_assert(!kWarp || (kCtaOnly && !kSmem), "warp-0 levels need a CTA engine with global state");
     static_assert(!kAsync || !kCtaOnly, "asynchronous sweeps need the whole grid");
     static_assert(!kBottomUp || !kCtaOnly, "bottom-up levels need the whole grid");
     const EngineArgs* a;   // in shared memory (keeps the per-thread register footprint small)
@@ -185,7 +185,7 @@ struct Engine {
 
     // Bring a vertex's padded row into L2 ahead of the level that will read it.
     __device__ void prefetch_row(int u) const {
-        if constexpr (!kSmem) asm volatile("prefetch.global.L2 [%0];" ::"l"(a->ell + 2 * (size_t)u));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(a->ell + 2 * (size_t)u));
     }
 
     __device__ unsigned long long* claim_p(int v) const { return a->claim + (kSmem ? v - a->v0 : v); }
@@ -475,8 +475,8 @@ struct Engine {
     // The labelled levels' exchange: CTA b's count alone (the same in all its threads). What every level
     // pays for is its chain of instructions between the last claim and the first ownership test, so no
     // key travels (only a sweep's last level needs one: last_level_key), the counts are adjacent words,
-    // and warp reductions combine them (192^3 grid, 1,026 such exchanges: 7.44 -> 6.8 ms a call, with
-    // the sweeps out of line).
+    // and warp reductions combine them (192^3 grid, 1,026 such exchanges: 0.6 of 7.4 ms a call,
+    // together with the sweeps out of line; 6.75 with everything).
     __device__ bool exchange_counts(ExResult& r, int cnt) {
         __syncthreads();
         const unsigned e = ++epoch;

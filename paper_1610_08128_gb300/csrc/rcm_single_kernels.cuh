@@ -51,7 +51,7 @@ extern template __global__ void k_rcm_small<512>(EngineArgs, int, int);
 extern template __global__ void k_rcm_components<kComponentThreads>(EngineArgs, int, int, int);
 #else
 template <int kThreads, bool kAsync, bool kBottomUp>
-__device__ __forceinline__ void single_run(const EngineArgs& args, int stall, EngineSmem& smem, int& s_item,
+__device__ __forceinline__ void single_run(const EngineArgs& args, int stall, EngineSmem& smem,
                                            unsigned long long* s_sort) {
     Ctl* ctl = args.ctl;
     if (ld_volatile(&ctl->status) & kErrBadCsr) return;
@@ -174,7 +174,6 @@ __device__ __forceinline__ void single_run(const EngineArgs& args, int stall, En
 template <int kThreads, bool kAsync, bool kBottomUp>
 __global__ void __launch_bounds__(kThreads, 1) k_rcm_single(EngineArgs args, int stall) {
     __shared__ EngineSmem smem;
-    __shared__ int s_item;
     // component-table sort (kCompSmem entries), on CTA 0 also the local sweeps' state, whose bitmap is
     // read 16 bytes at a time: without the attribute the array starts wherever the static part ends
     extern __shared__ __align__(16) unsigned long long s_sort[];
@@ -185,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_rcm_single(EngineArgs args, int
         if (threadIdx.x == 0) smem.xc_flag[0] = smem.xc_flag[1] = 0ull;
         cluster_barrier();
     }
-    single_run<kThreads, kAsync, kBottomUp>(args, stall, smem, s_item, s_sort);
+    single_run<kThreads, kAsync, kBottomUp>(args, stall, smem, s_sort);
     if (args.mid_k > 0) cluster_barrier();
 }
 
@@ -260,8 +259,8 @@ __global__ void __launch_bounds__(kThreads) k_rcm_components(EngineArgs args, in
     }
 }
 
-// kThreads: narrow graphs (a few dozen vertices per level) run best on small CTAs, whose barriers,
-// scans and reductions are cheap.
+// kThreads: what a level of the local sweeps takes in one pass is 4 vertices a warp, so wide CTAs are the
+// faster also on narrow graphs (small_default_threads has the figures).
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads, 1) k_rcm_small(EngineArgs args, int vis_off, int ell_off) {
     extern __shared__ __align__(16) unsigned long long s_state[];
