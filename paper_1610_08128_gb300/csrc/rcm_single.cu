@@ -298,8 +298,9 @@ rcm_status single_launch(int n, long long nnz, const rcm_options& o, SingleLaunc
         }
     }
     // narrow runs keep the frontier in a shared-memory cache of kCache ids
-    // default switch at the CTA width: for 512-thread CTAs it beat twice the width on every graph
-    // measured on GB300 (the 192^3 grid 7.40 against 7.64 ms, a 1000^2 grid 19.1 against 24.3 ms)
+    // default switch at the CTA width: half and twice of it cost more on some graphs than they save on others
+    // (GB300, 256 / 512 / 1,024: the 192^3 grid 6.73 / 6.73 / 7.03 ms, a 100^3 grid 2.70 / 2.67 / 3.24, a
+    // 1000^2 grid 13.8 / 12.35 / 12.28, a 1M-point 3-NN mesh 22.3 / 19.7 / 18.4)
     int narrow = o.narrow_threshold == 0 ? sl.threads : (o.narrow_threshold < 0 ? 0 : o.narrow_threshold);
     sl.narrow = std::min(narrow, kCache);
     // CTA 0's narrow levels in shared memory: where its CTA has the SM to itself and no middle tier
@@ -307,11 +308,11 @@ rcm_status single_launch(int n, long long nnz, const rcm_options& o, SingleLaunc
     // (nor on patterns dense enough for bottom-up levels: they have few levels, and wide ones)
     sl.local = sl.threads == 512 && !sl.hybrid && sl.narrow > 1 && sl.mid_k == 0 && sl.blocks <= di.sms;
     sl.limit_ns = o.spin_limit_ns > 0 ? o.spin_limit_ns : 20000000000LL;
-    // label during every sweep by default on a wide grid: there a labelled level is cheaper than a
-    // levels-only one (GB300, 152 CTAs: the 192^3 grid 7.08 against 7.43 ms, a 1000^2 grid 17.7
-    // against 18.6 ms, the 1.2M-point mesh 24.5 against 25.4 ms). On a few CTAs the extra work of
-    // a labelled first sweep costs more than it saves (one cluster of 6: a 100^3 grid 8.6 against
-    // 6.8 ms). Asynchronous sweeps are levels-only.
+    // label during every sweep by default on a wide grid: there a narrow labelled level, in CTA 0's shared
+    // memory, is cheaper than a levels-only one (GB300, 152 CTAs: a 1000^2 grid 12.35 against 13.5 ms, a
+    // 1M-point 3-NN mesh 19.7 against 20.3, a 100^3 grid 2.67 against 2.75; the 192^3 grid, nearly all
+    // wide levels, 6.70 against 6.66). On a few CTAs the extra work of a labelled first sweep costs more than
+    // it saves (one cluster of 6: a 100^3 grid 8.3 against 6.5 ms). Asynchronous sweeps are levels-only.
     sl.fused = o.fused_sweeps < 0 ? 0 : o.fused_sweeps == 1 ? 1 : o.fused_sweeps == 2 ? 2
              : (sl.async || sl.blocks < kLabelEverySweepBlocks) ? 1 : 2;
     // hub graphs (a vertex of more than kHubDegree neighbours) take a lower switch and levels-only
