@@ -163,7 +163,7 @@ typedef struct {
                                   serial); one union-find pass more on a connected graph. Same
                                   result. -1 = off; 0 = decided on the device: where the rows average
                                   fewer than 3.2 neighbours that first sweep gives up for the table
-                                  if its 64th level is narrow (off on a cluster)                    */
+                                  if its 32nd level is narrow (off on a cluster)                    */
 } rcm_options;
 
 /* Statistics of one ordering (filled by rcm_order_ex when requested). */

@@ -24,10 +24,10 @@ constexpr int kHubShare = 1024;
 // one part while everything else waits (1.2M-point mesh in 20 strips 9.6 ms with it, 8.0 without); the
 // component table costs a pass of union-find, 0.3 ms per million vertices. Trees, cubic and other sparse random
 // graphs are as sparse, but connected and low, and the table is lost on them. So the probe runs, and gives
-// up for the table where level kProbeLevels is still narrow (0.1 ms of the strips' 8.0; a 20,000-vertex tree
-// 0.64 ms, and 0.94 with 32 levels, where it gives up).
+// up for the table where level kProbeLevels is still narrow and 3/4 of the vertices are not reached yet
+// (0.05 ms of the strips' 8.0; a 50,000-vertex cubic graph, which finishes it, 0.24 ms, and 0.43 with the table).
 constexpr int kPartsDegree = 32;
-constexpr int kProbeLevels = 64;
+constexpr int kProbeLevels = 32;
 // Levels of up to this many vertices are one CTA's work: a 50,000-vertex path 72 ms on 256 threads, 84 on
 // CTA 0 of the grid; a 260^2 grid with its edges halved 5.6 and 5.1.
 constexpr int kThinLevel = 8;

@@ -77,7 +77,7 @@ NARROW = {
     "path_5k": lambda: synth.path(5000, seed=9),                       # connected: the table has one entry
     "road": lambda: halved((70, 70), 18),                              # connected, and not that thin
     "strips": lambda: synth.knn_mesh(20_000, 2, 10, regions=6),
-    "paths": lambda: beside([synth.path(n, seed=n) for n in (65, 64, 63, 2000, 3000, 3001, 66, 130)], 11),
+    "paths": lambda: beside([synth.path(n, seed=n) for n in (33, 32, 31, 34, 65, 64, 63, 66, 130, 2000, 3000, 3001)], 11),
     "just_under": lambda: beside([cubic(20_000, 12), cubic(20_000, 13)], 14),
     # the first start vertex (least degree, least id) lies on a path beside wide parts
     "path_first": lambda: beside([cubic(20_000, 15), synth.path(1500, seed=16)], 17),
