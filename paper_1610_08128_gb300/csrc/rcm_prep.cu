@@ -83,8 +83,9 @@ __global__ void k_degree_validate(int n, int nnz, const int* __restrict__ rowptr
             const int ra = __shfl_sync(0xffffffffu, a, src), rb = __shfl_sync(0xffffffffu, b, src);
             const int rlo = __shfl_sync(0xffffffffu, lo, src), rhi = __shfl_sync(0xffffffffu, hi, src);
             int c = 0;
-            for (int k = ra + lane; k < rb; k += 32) {
-                const int w = __ldg(colidx + k);
+            const int* entries = colidx + ra;  // (counted from the row's start: offsets near 2^31 do not wrap)
+            for (unsigned k = lane; k < (unsigned)(rb - ra); k += 32) {
+                const int w = __ldg(entries + k);
                 bad |= w < rlo || w >= rhi;
                 c += w != row ? 1 : 0;
             }
@@ -97,10 +98,12 @@ __global__ void k_degree_validate(int n, int nnz, const int* __restrict__ rowptr
         }
         {
             // the others by their thread, 8 entries at a time, all loaded before the first is looked at
-            for (int k = a; k < b && b - a <= kDegLong; k += 8) {
+            const int len = b - a;
+            const int* entries = colidx + a;
+            for (int k = 0; k < len && len <= kDegLong; k += 8) {
                 int w[8];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) w[t] = k + t < b ? __ldg(colidx + k + t) : v;
+                for (int t = 0; t < 8; ++t) w[t] = k + t < len ? __ldg(entries + k + t) : v;
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
                     bad |= w[t] < lo || w[t] >= hi;
@@ -184,12 +187,12 @@ __global__ void k_sort_rows_big(int n, const int* __restrict__ rowptr, const int
         const int a = rowptr[v], b = rowptr[v + 1];
         if (b - a > kWarpRowMax) continue;
         int m = 0;
-        for (int k0 = a; k0 < b; k0 += 32) {
+        for (int k0 = 0; k0 < b - a; k0 += 32) {
             const int k = k0 + lane;
-            const int w = k < b ? colidx[k] : v;
+            const int w = k < b - a ? colidx[a + k] : v;
             const bool keep = w != v;
             const unsigned bal = __ballot_sync(0xffffffffu, keep);
-            if (keep) ws[m + __popc(bal & ((1u << lane) - 1u))] = row_key(deg, w, k - a, by_degree);
+            if (keep) ws[m + __popc(bal & ((1u << lane) - 1u))] = row_key(deg, w, k, by_degree);
             m += __popc(bal);
         }
         int P = 1;
@@ -212,9 +215,9 @@ __global__ void k_sort_rows_big(int n, const int* __restrict__ rowptr, const int
         if (P > kBigRowSmem) continue;
         if (threadIdx.x == 0) s_m = 0;
         __syncthreads();
-        for (int k = a + threadIdx.x; k < b; k += blockDim.x) {
-            const int w = colidx[k];
-            if (w != v) s_keys[atomicAdd(&s_m, 1)] = row_key(deg, w, k - a, by_degree);
+        for (unsigned k = threadIdx.x; k < (unsigned)(b - a); k += blockDim.x) {
+            const int w = colidx[a + k];
+            if (w != v) s_keys[atomicAdd(&s_m, 1)] = row_key(deg, w, (int)k, by_degree);
         }
         __syncthreads();
         for (int i = m + threadIdx.x; i < P; i += blockDim.x) s_keys[i] = kKeyMax;
@@ -246,9 +249,9 @@ __global__ void k_sort_rows_big(int n, const int* __restrict__ rowptr, const int
         const int a = rowptr[v], b = rowptr[v + 1];
         if (threadIdx.x == 0) s_m = 0;
         __syncthreads();
-        for (int k = a + threadIdx.x; k < b; k += blockDim.x) {
-            const int w = colidx[k];
-            if (w != v) scratch[atomicAdd(&s_m, 1)] = row_key(deg, w, k - a, by_degree);
+        for (unsigned k = threadIdx.x; k < (unsigned)(b - a); k += blockDim.x) {
+            const int w = colidx[a + k];
+            if (w != v) scratch[atomicAdd(&s_m, 1)] = row_key(deg, w, (int)k, by_degree);
         }
         __syncthreads();
         for (int i = m + threadIdx.x; i < P; i += blockDim.x) scratch[i] = kKeyMax;
@@ -296,22 +299,25 @@ __global__ void k_bw_rows(int n, const int* __restrict__ rowptr, const int* __re
             a = rowptr[v];
             b = rowptr[v + 1];
         }
-        if (b - a <= kBwLong) {
-            for (int k = a; k < b; k += 8) {
+        const int len = b - a;
+        const int* entries = colidx + a;  // (counted from the row's start: offsets near 2^31 do not wrap)
+        if (len <= kBwLong) {
+            for (int k = 0; k < len; k += 8) {
                 int w[8];
 #pragma unroll
-                for (int t = 0; t < 8; ++t) w[t] = k + t < b ? colidx[k + t] : v;
+                for (int t = 0; t < 8; ++t) w[t] = k + t < len ? entries[k + t] : v;
 #pragma unroll
                 for (int t = 0; t < 8; ++t) w[t] = __ldg(pos + w[t]);
 #pragma unroll
                 for (int t = 0; t < 8; ++t) f = min(f, w[t]);
             }
         }
-        for (unsigned m = __ballot_sync(0xffffffffu, b - a > kBwLong); m; m &= m - 1) {
+        for (unsigned m = __ballot_sync(0xffffffffu, len > kBwLong); m; m &= m - 1) {
             const int src = __ffs(m) - 1;
             const int ra = __shfl_sync(0xffffffffu, a, src), rb = __shfl_sync(0xffffffffu, b, src);
             int least = kIntMax;
-            for (int k = ra + lane; k < rb; k += 32) least = min(least, __ldg(pos + colidx[k]));
+            const int* row = colidx + ra;
+            for (unsigned k = lane; k < (unsigned)(rb - ra); k += 32) least = min(least, __ldg(pos + row[k]));
             least = __reduce_min_sync(0xffffffffu, least);
             if (lane == src) f = min(f, least);
         }

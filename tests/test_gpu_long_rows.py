@@ -105,3 +105,27 @@ def test_components_beyond_the_bitmap(rcm):
     got, stats = rcm.order(device(g.rowptr), device(g.colidx), with_stats=True)
     assert stats["components"] == 408
     assert np.array_equal(got.cpu().numpy(), oracle.rcm(g.n, g.rowptr, g.colidx))
+
+
+@pytest.mark.parametrize("last", [63, 99, 5000])
+def test_bandwidth_with_the_most_entries(rcm, last):
+    """2^31 - 1 stored entries: the offsets of the last rows are within a row's length of the largest int32."""
+    free, _ = torch.cuda.mem_get_info()
+    if free < 60 << 30:
+        pytest.skip("needs 60 GB")
+    n, nnz = 1 << 25, (1 << 31) - 1
+    buf = torch.randint(0, n, (nnz + 1,), dtype=torch.int32, device="cuda")
+    rowptr = torch.clamp(torch.arange(n + 1, device="cuda") * 64, max=nnz - last)
+    rowptr[n] = nnz
+    first = (nnz - last) // 64  # rows before this one have 64 entries
+    buf[rowptr[n - 1]:nnz] = n - 2  # the last row reaches back by one, and by more in its last entry alone
+    buf[nnz - 1] = 7
+    beta = torch.arange(n, device="cuda")
+    beta[:first] -= torch.minimum(beta[:first], buf[:64 * first].view(first, 64).amin(1).long())
+    rest = buf[64 * first:nnz - last].long()
+    beta[first:] = 0
+    if len(rest):
+        beta[first] = max(0, first - int(rest.min()))
+    beta[n - 1] = n - 1 - 7
+    got = rcm.bandwidth_profile(rowptr.int(), buf[:nnz], torch.arange(n, dtype=torch.int32, device="cuda"))
+    assert got == (int(beta.max()), int(beta.sum()))
